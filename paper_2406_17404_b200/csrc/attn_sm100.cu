@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(at_threads(AT_SPLIT), 1) tree_attention_tc_ker
     float* piece_o = reinterpret_cast<float*>(base_ptr + AT_TILE);          // [row][AT_PIECE_STRIDE], over the K/V ring once it is idle
 
     if (warp == AT_W_COPY) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ------------------------------------------------ TMA producer
             int g = 0, e = 0;
             bool ok = true;
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(at_threads(AT_SPLIT), 1) tree_attention_tc_ker
             if (!waited) pdl_wait();
         }
     } else if (warp == AT_W_MMA) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ------------------------------------------------ MMA issuer
             // S = Q.K^T: both K-major from shared memory, 128 x 128.  O += P.V: P from TMEM, V MN-major, 128 x 128.
             const uint32_t idesc_qk = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(AT_KEYS >> 3) << 17) | ((uint32_t)(AT_ROWS >> 4) << 24);

@@ -44,6 +44,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// True in one lane of a converged warp.  The instructions that one thread issues for a CTA (TMA copies, MMAs, commits)
+// take their operands from uniform registers: behind elect.sync the compiler knows that a single lane is active, behind
+// `lane == 0` it prepares every operand for a divergent warp.  Measured with clock stamps in the projection kernel: 4 MMAs
+// and a commit took 590 cycles to issue behind `lane == 0`, 222 behind elect.sync, and a whole role loop behind one
+// elect.sync is faster than an elect.sync per use (a K step: 950 cycles whatever its size, then 510 for small ones).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
+}
+
 // Data that is read once per step and is far larger than L2 (weights, cache tiles) is loaded with an
 // evict-first policy so that it does not push out what is reused between kernels.
 __device__ __forceinline__ uint64_t l2_evict_first_policy() {
