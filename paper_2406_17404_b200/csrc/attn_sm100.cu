@@ -197,12 +197,7 @@ __device__ __forceinline__ void store4_split(__nv_bfloat16* hi, __nv_bfloat16* l
         *reinterpret_cast<uint2*>(lo) = make_uint2(pack_bf16(a - bf16_round(a), b - bf16_round(b)),
                                                    pack_bf16(c - bf16_round(c), d - bf16_round(d)));
 }
-// Distributed shared memory: the address of `local` (a shared::cta address) in CTA `rank` of the cluster, and loads from it.
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-    return r;
-}
+// Loads from distributed shared memory.
 __device__ __forceinline__ float ld_cluster(uint32_t addr) {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
@@ -213,11 +208,6 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // 128-bit (lo, hi) shifts by 0..127 bits; the left shift fills the vacated low bits with ones.
 __device__ __forceinline__ void shr128(uint64_t& lo, uint64_t& hi, int n) {
     if (n == 0) return;
