@@ -247,12 +247,11 @@ size_t carve(const trj_model_cfg& c, void* ws, trj_ctx* ctx) {
     // a prefill chunk's pieces are the sequences of one attention launch
     const size_t attn_bytes = trj_tree_attention_workspace(rows, std::max(c.max_batch, PREFILL_MAX_SUB), c.n_heads, c.head_dim, c.max_seq);
     char* attn_ws = cv.take<char>(attn_bytes);
-    // every row count a call may bring (the K split, hence the space for partial sums, is not monotone in it)
-    size_t gemm_bytes = 256;
-    for (auto nk : {std::pair<int, int>{QKV, c.d_model}, {c.d_model, HD}, {2 * c.d_ff, c.d_model},
-                    {c.d_model, c.d_ff}, {c.vocab, c.d_model}})
-        for (int m = 1; m <= rows; ++m)
-            gemm_bytes = std::max(gemm_bytes, gemm_tc_workspace(m, nk.first, nk.second));
+    size_t gemm_bytes = 256;                                 // fp32 models have no partial sums
+    if (c.dtype == TRJ_BF16)
+        for (auto nk : {std::pair<int, int>{QKV, c.d_model}, {c.d_model, HD}, {2 * c.d_ff, c.d_model},
+                        {c.d_model, c.d_ff}, {c.vocab, c.d_model}})
+            gemm_bytes = std::max(gemm_bytes, gemm_tc_max_workspace(rows, nk.first, nk.second));
     char* gemm_ws = cv.take<char>(gemm_bytes);
     int32_t* chain_depth = cv.take<int32_t>(PREFILL_CHUNK);
     int32_t* prefill_geo = cv.take<int32_t>(2 * PREFILL_MAX_SUB + 4);   // piece lengths, {0, m}, piece row offsets

@@ -135,6 +135,7 @@ cudaError_t launch_gemm_simt(const void* x, const void* x_lo, const void* w, flo
 bool gemm_tc_supported(const void* x, const void* x_lo, const void* w, const float* y, int32_t M, int32_t N, int32_t K,
                        int32_t dtype);
 size_t gemm_tc_workspace(int32_t M, int32_t N, int32_t K);
+size_t gemm_tc_max_workspace(int32_t max_rows, int32_t N, int32_t K);      // ... of any row count up to max_rows
 cudaError_t launch_gemm_tc(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N, int32_t K,
                            void* workspace, cudaStream_t st, Parts* parts, const WeightPrefetch* ahead = nullptr,
                            int* status = nullptr, const TopTable* top = nullptr);
