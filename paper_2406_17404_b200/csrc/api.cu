@@ -177,6 +177,7 @@ struct trj_ctx {
     float* h; float* y; float* logits;
     void* x; void* x_lo; void* q; void* act; void* act_lo;   // *_lo: low halves of split bf16 activations
     double* inv_freq;
+    Rotary rot;            // of the rows of the latest forward
     int sm_count;          // SMs of the device the context lives on
     void* argmax_ws; void* attn_ws; size_t attn_ws_bytes; void* gemm_ws; size_t gemm_ws_bytes;
     // chain-tree tables for prefill and the staging area of trj_step_host (device)
@@ -243,6 +244,8 @@ size_t carve(const trj_model_cfg& c, void* ws, trj_ctx* ctx) {
     char* act = cv.take<char>((size_t)rows * c.d_ff * es);
     char* act_lo = cv.take<char>((size_t)rows * c.d_ff * es);
     double* inv_freq = cv.take<double>(c.head_dim / 2);
+    float* rot_table = cv.take<float>((size_t)rows * c.head_dim);
+    int2* rot_row_at = cv.take<int2>(rows);
     char* argmax_ws = cv.take<char>(argmax_workspace_bytes(step_rows, c.max_batch));
     // a prefill chunk's pieces are the sequences of one attention launch
     const size_t attn_bytes = trj_tree_attention_workspace(rows, std::max(c.max_batch, PREFILL_MAX_SUB), c.n_heads, c.head_dim, c.max_seq);
@@ -268,7 +271,7 @@ size_t carve(const trj_model_cfg& c, void* ws, trj_ctx* ctx) {
     if (ctx) {
         ctx->h = h; ctx->y = y; ctx->logits = logits; ctx->x = x; ctx->q = q; ctx->act = act;
         ctx->x_lo = c.dtype == TRJ_BF16 ? x_lo : nullptr; ctx->act_lo = c.dtype == TRJ_BF16 ? act_lo : nullptr;
-        ctx->inv_freq = inv_freq; ctx->argmax_ws = argmax_ws; ctx->attn_ws = attn_ws; ctx->attn_ws_bytes = attn_bytes;
+        ctx->inv_freq = inv_freq; ctx->rot = Rotary{rot_table, rot_row_at}; ctx->argmax_ws = argmax_ws; ctx->attn_ws = attn_ws; ctx->attn_ws_bytes = attn_bytes;
         ctx->gemm_ws = gemm_ws; ctx->gemm_ws_bytes = gemm_bytes;
         ctx->chain_depth = chain_depth; ctx->chain_anc = chain_anc; ctx->prefill_geo = prefill_geo;
         ctx->chunk_row_off = chunk_row_off; ctx->unit_row_off = unit_row_off;
@@ -335,7 +338,7 @@ void prof_end(trj_ctx* ctx, cudaStream_t st) {
 // piece, every piece a chain below all rows before it.
 struct StepArgs {
     void* k_cache; void* v_cache; int32_t b0; Batch bt;
-    const int32_t* tokens; const int32_t* depth; const uint64_t* anc; int32_t anc_words;
+    const int32_t* depth; const uint64_t* anc; int32_t anc_words;
     int32_t lm_first, lm_rows; const SubChunks* pieces;
     int32_t lm_mode;   // 0: logits; 1: logits and the arg-max candidates of the epilogue; 2: the candidates only
 };
@@ -390,8 +393,8 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
                                                         c.rms_eps, st));
             LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
                                           ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
-            LAUNCH(PROF_ROPE, launch_rope_kv_write(pr, ctx->inv_freq, a.depth, bt, ctx->q, k_slab, v_slab, c.dtype,
-                                                   c.n_heads, Hkv, c.head_dim, c.max_seq, st));
+            LAUNCH(PROF_ROPE, launch_rope_kv_write(pr, ctx->rot, ctx->inv_freq, a.depth, bt, ctx->q, k_slab, v_slab, c.dtype, c.n_heads, Hkv,
+                                                   c.head_dim, c.max_seq, st));
             // inside the decoder the attention result reaches the output projection as a bf16 pair, like every
             // other projection input
             if (!pieces) {
@@ -431,9 +434,9 @@ trj_status forward(trj_ctx* ctx, void* k_cache, void* v_cache, int32_t b0, const
                    int32_t lm_first, int32_t lm_rows, cudaStream_t st, const SubChunks* pieces = nullptr, int32_t lm_mode = 0) {
     ChainScope chain;                        // the embedding below is the chain's fence
     const trj_model_cfg& c = ctx->cfg;
-    LAUNCH(PROF_ELEMENTWISE, launch_embed(ctx->embed, c.dtype, tokens, ctx->h, bt.rows_total, c.d_model, st));
+    LAUNCH(PROF_ELEMENTWISE, launch_embed(ctx->embed, c.dtype, tokens, ctx->h, c.d_model, ctx->inv_freq, c.head_dim, depth, bt, ctx->rot, st));
     Parts pr{nullptr, 1, 0};                 // result of the latest projection, possibly in split-K pieces
-    const StepArgs a{k_cache, v_cache, b0, bt, tokens, depth, anc, anc_words, lm_first, lm_rows, pieces, lm_mode};
+    const StepArgs a{k_cache, v_cache, b0, bt, depth, anc, anc_words, lm_first, lm_rows, pieces, lm_mode};
     return run_segments(ctx, a, 0, 2 * c.n_layers + 1, pr, false, st);
 }
 
@@ -688,7 +691,8 @@ extern "C" trj_status trj_tp_begin(trj_ctx* ctx, void* k_cache, void* v_cache, c
     cudaStream_t st = (cudaStream_t)stream;
     ChainScope chain;
     ctx->tp = trj_ctx::TpStep{};
-    LAUNCH(PROF_ELEMENTWISE, launch_embed(ctx->embed, ctx->cfg.dtype, tokens, ctx->h, rows_total, ctx->cfg.d_model, st));
+    LAUNCH(PROF_ELEMENTWISE, launch_embed(ctx->embed, ctx->cfg.dtype, tokens, ctx->h, ctx->cfg.d_model, ctx->inv_freq, ctx->cfg.head_dim, depth,
+                                          Batch{seq_len, row_off, B, rows_total, max_rows, max_len}, ctx->rot, st));
     ctx->tp.open = true; ctx->tp.next = 0; ctx->tp.k_cache = k_cache; ctx->tp.v_cache = v_cache;
     ctx->tp.bt = Batch{seq_len, row_off, B, rows_total, max_rows, max_len};
     ctx->tp.tokens = tokens; ctx->tp.parent = parent; ctx->tp.depth = depth; ctx->tp.anc = anc; ctx->tp.anc_words = anc_words;
@@ -704,7 +708,7 @@ extern "C" trj_status trj_tp_segment(trj_ctx* ctx, int32_t segment, void* stream
     cudaStream_t st = (cudaStream_t)stream;
     ChainScope chain;
     const trj_ctx::TpStep& t = ctx->tp;
-    const StepArgs a{t.k_cache, t.v_cache, 0, t.bt, t.tokens, t.depth, t.anc, t.anc_words, 0, t.bt.rows_total, nullptr, 0};
+    const StepArgs a{t.k_cache, t.v_cache, 0, t.bt, t.depth, t.anc, t.anc_words, 0, t.bt.rows_total, nullptr, 0};
     // what the previous segment left, summed over the ranks by the caller, sits in the exchange buffer
     Parts pr = segment == 0 ? Parts{nullptr, 1, 0} : whole(ctx->y);
     trj_status s = run_segments(ctx, a, segment, segment + 1, pr, segment + 1 < n_seg, st);

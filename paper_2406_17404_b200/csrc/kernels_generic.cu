@@ -64,10 +64,10 @@ __device__ __forceinline__ float4 parts_at4(const Parts& p, size_t i4) {
     return v;
 }
 
-// Same for four consecutive values.  The pieces are requested eight at a time before any is added, so the
+// Same for four consecutive values.  The pieces are requested BATCH at a time before any is added, so the
 // loads overlap; the additions keep the order of the pieces.
+template <int BATCH>
 __device__ __forceinline__ float4 parts_at4_batched(const Parts& p, size_t i4) {
-    constexpr int BATCH = 8;
     float4 v = reinterpret_cast<const float4*>(p.ptr)[i4];
     for (int s0 = 1; s0 < p.splits; s0 += BATCH) {
         float4 b[BATCH];
@@ -88,10 +88,21 @@ __device__ __forceinline__ int seq_of_row(const int32_t* row_off, int B, int row
     return b;
 }
 
+// Sine and cosine of a rotary angle: formed in fp64 (positions reach thousands of radians) and reduced to [-pi, pi] there;
+// sin/cos of the reduced angle in fp32 are then accurate to ~1e-7.
+__device__ __forceinline__ void rotation(double ang, float& sn, float& cs) {
+    const double red = ang - 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
+    sincosf((float)red, &sn, &cs);
+}
+
 // ---------------------------------------------------------------- embedding
+// With a table (`rot`) it also works out, once per forward, what the rotary kernel of every layer needs of a row: the cosines
+// and sines of its position and where its K/V rows go.
 template <typename T>
 __global__ void embed_kernel(const T* __restrict__ embed, const int32_t* __restrict__ tokens,
-                             float* __restrict__ h, int d) {
+                             float* __restrict__ h, int d, const double* __restrict__ inv_freq, int half,
+                             const int32_t* __restrict__ depth, const int32_t* __restrict__ seq_len,
+                             const int32_t* __restrict__ row_off, int B, float* __restrict__ rot, int2* __restrict__ row_at) {
     pdl_wait();                                  // the chain's fence: everything enqueued earlier is complete
     pdl_launch_dependents();                     // before any later kernel of the chain may start
     TRJ_TL_DECL; TRJ_TL_BEGIN(TRJ_TL_EMBED);
@@ -113,14 +124,28 @@ __global__ void embed_kernel(const T* __restrict__ embed, const int32_t* __restr
     } else {
         for (int c = threadIdx.x; c < d; c += blockDim.x) h[(size_t)row * d + c] = to_f(src[c]);
     }
+    if (rot) {
+        const int b = seq_of_row(row_off, B, row);
+        const int len = seq_len[b];
+        for (int i = threadIdx.x; i < half; i += blockDim.x) {
+            float sn, cs;
+            rotation((double)(len + depth[row]) * inv_freq[i], sn, cs);
+            rot[(size_t)row * 2 * half + i] = cs;
+            rot[(size_t)row * 2 * half + half + i] = sn;
+        }
+        if (threadIdx.x == 0) row_at[row] = make_int2(b, len + row - row_off[b]);
+    }
     TRJ_TL_END(TRJ_TL_EMBED);
 }
 
 // ---------------------------------------------------------------- residual add + RMSNorm
 // One CTA per row.  h += add (summing the split-K pieces of `add` on the way), x = rmsnorm(h) * gain.
-// Fast path: d % 4 == 0 and d <= 4 * RMS_THREADS * RMS_CHUNKS; the row lives in registers between the two phases.
-constexpr int RMS_THREADS = 1024;             // many loads in flight: the row and its split-K pieces come from L2
-constexpr int RMS_CHUNKS = 2;
+// Fast path: d % 4 == 0 and d <= RMS_MAX_D; the row lives in registers between the two phases.  Up to one row per SM a
+// row takes 1024 threads, for many loads in flight (the row and its split-K pieces come from L2); more rows take 256 threads
+// each, so that eight CTAs share an SM and one's barriers overlap the others' loads (1024 rows of 4096: 22.5 -> 11.6 us, 64 MB
+// from and to L2; 320 rows with two pieces 8.6 -> 7.0 us).
+constexpr int RMS_MAX_D = 8192;
+constexpr int RMS_FEW_ROWS = 148, RMS_FEW_ROWS_THREADS = 1024;
 
 __device__ __forceinline__ float block_sum(float v, float* red) {
     v = warp_sum(v);
@@ -155,35 +180,62 @@ __device__ __forceinline__ void store_split4<__nv_bfloat16>(__nv_bfloat16* hi, _
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(RMS_THREADS) add_rmsnorm_vec_kernel(float* __restrict__ h, const Parts add,
-                                                                     const float* __restrict__ gain, T* __restrict__ x,
-                                                                     T* __restrict__ x_lo, int d, float eps) {
+template <typename T, int THREADS, int CHUNKS>
+__global__ void __launch_bounds__(THREADS) add_rmsnorm_vec_kernel(float* __restrict__ h, const Parts add,
+                                                                 const float* __restrict__ gain, T* __restrict__ x,
+                                                                 T* __restrict__ x_lo, int d, float eps) {
     pdl_prologue();
     TRJ_TL_DECL; TRJ_TL_BEGIN(TRJ_TL_RMSNORM);
     __shared__ float red[32];
     const int row = blockIdx.x, n4 = d >> 2;
-    float4 v[RMS_CHUNKS];
+    float4 v[CHUNKS];
     float ss = 0.f;
+    if constexpr (THREADS == RMS_FEW_ROWS_THREADS) {
+        // one load after the other: requesting them together makes this kernel faster (4.0 -> 3.7 us) and the step it sits
+        // in slower (33 rows 3.13 -> 3.15 ms): the next projection's weight ring is filling at the same time
 #pragma unroll
-    for (int k = 0; k < RMS_CHUNKS; ++k) {
-        const int j = threadIdx.x + k * RMS_THREADS;
-        if (j < n4) {
-            v[k] = reinterpret_cast<const float4*>(h + (size_t)row * d)[j];
-            if (add.ptr) {
-                // one piece after the other: requesting them together was measured slower inside the step (4.2 against
-                // 3.9 us), where the next projection's weight ring is filling at the same time
-                const float4 a = parts_at4(add, (size_t)row * n4 + j);
-                v[k].x += a.x; v[k].y += a.y; v[k].z += a.z; v[k].w += a.w;
-                reinterpret_cast<float4*>(h + (size_t)row * d)[j] = v[k];
+        for (int k = 0; k < CHUNKS; ++k) {
+            const int j = threadIdx.x + k * THREADS;
+            if (j < n4) {
+                v[k] = reinterpret_cast<const float4*>(h + (size_t)row * d)[j];
+                if (add.ptr) {
+                    const float4 a = parts_at4(add, (size_t)row * n4 + j);
+                    v[k].x += a.x; v[k].y += a.y; v[k].z += a.z; v[k].w += a.w;
+                    reinterpret_cast<float4*>(h + (size_t)row * d)[j] = v[k];
+                }
+                ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
             }
-            ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
         }
+    } else {
+        float4 a[CHUNKS];
+#pragma unroll
+        for (int k = 0; k < CHUNKS; ++k) {
+            const int j = threadIdx.x + k * THREADS;
+            if (j < n4) v[k] = reinterpret_cast<const float4*>(h + (size_t)row * d)[j];
+        }
+        if (add.ptr) {
+#pragma unroll
+            for (int k = 0; k < CHUNKS; ++k) {
+                const int j = threadIdx.x + k * THREADS;
+                if (j < n4) a[k] = parts_at4(add, (size_t)row * n4 + j);
+            }
+#pragma unroll
+            for (int k = 0; k < CHUNKS; ++k) {
+                const int j = threadIdx.x + k * THREADS;
+                if (j < n4) {
+                    v[k].x += a[k].x; v[k].y += a[k].y; v[k].z += a[k].z; v[k].w += a[k].w;
+                    reinterpret_cast<float4*>(h + (size_t)row * d)[j] = v[k];
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < CHUNKS; ++k)
+            if (threadIdx.x + k * THREADS < n4) ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
     }
     const float inv = rsqrtf(block_sum(ss, red) / (float)d + eps);
 #pragma unroll
-    for (int k = 0; k < RMS_CHUNKS; ++k) {
-        const int j = threadIdx.x + k * RMS_THREADS;
+    for (int k = 0; k < CHUNKS; ++k) {
+        const int j = threadIdx.x + k * THREADS;
         if (j < n4) {
             const float4 g = reinterpret_cast<const float4*>(gain)[j];
             store_split4<T>(x, x_lo, (size_t)row * d + 4 * j,
@@ -324,59 +376,17 @@ __global__ void __launch_bounds__(SF_THREADS) gemm_small_f32_kernel(const float*
 }
 
 // ---------------------------------------------------------------- rotary embedding + K/V append
+// Two kernels, both bound by the chain of loads and not by bytes.  Few rows: a thread takes a head's q, k and v (18 loads of
+// split-K pieces in flight) in a few fat CTAs, and works out its rotations ahead of the wait, where they cost nothing.  Many
+// rows: each layer and head working out the same rotations again does cost (1024 rows of the 7B shape: 45 us a layer), so the
+// embedding kernel leaves them in a table and a thread takes one head of q, k or v (26 us).  At 33 rows the table is the slower
+// way: 3.18 against 3.15 ms a step, its loads come after the wait.
+constexpr int ROPE_THREADS = 256;           // 16 heads of 128 dimensions
+constexpr int ROPE_FEW_ROWS = 148;
+// Four consecutive dimensions and the four they are rotated with per thread (head_dim / 2 a multiple of 4): 16-byte loads of
+// the projection pieces, 8-byte (bf16) or 16-byte (fp32) stores.  One CTA covers heads_per_cta heads of a row.
 template <typename T>
-__global__ void rope_kv_write_kernel(const Parts qkv, const double* __restrict__ inv_freq,
-                                     const int32_t* __restrict__ depth, const int32_t* __restrict__ seq_len,
-                                     const int32_t* __restrict__ row_off, int B, T* __restrict__ q_out,
-                                     T* __restrict__ k_slab, T* __restrict__ v_slab, int H, int Hkv, int D, int max_seq) {
-    pdl_launch_dependents();
-    // geometry and the rotation of this thread's first element do not depend on the projection: have them
-    // ready before waiting for it
-    const int row = blockIdx.x, hh = blockIdx.y;
-    const int b = seq_of_row(row_off, B, row);
-    const int local = row - row_off[b];
-    const int pos = seq_len[b] + depth[row];
-    const int half = D >> 1, HD = H * D, KD = Hkv * D;
-    const bool has_kv = hh < Hkv;                            // this CTA also handles K/V head hh
-    const size_t src = (size_t)row * (HD + 2 * KD) + hh * D; // flat index of query head hh in the projection result
-    const size_t cache_row = (((size_t)b * Hkv + hh) * max_seq + seq_len[b] + local) * D;
-    auto rotation = [&](int i, float& sn, float& cs) {
-        // angle in fp64 (positions reach thousands of radians), reduced to [-pi, pi] there; sin/cos of the reduced
-        // angle in fp32 are then accurate to ~1e-7
-        const double ang = (double)pos * inv_freq[i];
-        const double red = ang - 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
-        sincosf((float)red, &sn, &cs);
-    };
-    float sn = 0.f, cs = 1.f;
-    if ((int)threadIdx.x < half) rotation(threadIdx.x, sn, cs);
-    pdl_wait();
-    for (int i = threadIdx.x; i < half; i += blockDim.x) {
-        if (i != (int)threadIdx.x) rotation(i, sn, cs);
-        // all loads first: the stores below could alias them as far as the compiler knows
-        float qa = 0.f, qb = 0.f, ka = 0.f, kb = 0.f, va = 0.f, vb = 0.f;
-        for (int s = 0; s < qkv.splits; ++s) {               // six independent loads per split-K piece
-            const float* piece = qkv.ptr + (size_t)s * qkv.stride + src + i;
-            qa += piece[0];      qb += piece[half];
-            if (has_kv) {
-                ka += piece[HD];      kb += piece[HD + half];
-                va += piece[HD + KD]; vb += piece[HD + KD + half];
-            }
-        }
-        q_out[(size_t)row * HD + hh * D + i] = from_f<T>(qa * cs - qb * sn);
-        q_out[(size_t)row * HD + hh * D + i + half] = from_f<T>(qb * cs + qa * sn);
-        if (!has_kv || !TRJ_DEBUG_CHECK((unsigned)(seq_len[b] + local) < (unsigned)max_seq, DBG_ROPE_ROW)) continue;
-        k_slab[cache_row + i] = from_f<T>(ka * cs - kb * sn);
-        k_slab[cache_row + i + half] = from_f<T>(kb * cs + ka * sn);
-        v_slab[cache_row + i] = from_f<T>(va);
-        v_slab[cache_row + i + half] = from_f<T>(vb);
-    }
-}
-
-// Four consecutive dimensions per thread (head_dim / 2 a multiple of 4): 16-byte loads of the projection pieces,
-// 8-byte (bf16) or 16-byte (fp32) stores.  One CTA covers heads_per_cta heads of a row (at most ROPE_THREADS threads).
-constexpr int ROPE_THREADS = 256;           // a few fat CTAs (16 heads of 128 each) measured faster than many thin ones
-template <typename T>
-__global__ void __launch_bounds__(ROPE_THREADS) rope_kv_write_vec_kernel(const Parts qkv, const double* __restrict__ inv_freq,
+__global__ void __launch_bounds__(ROPE_THREADS) rope_kv_write_few_kernel(const Parts qkv, const double* __restrict__ inv_freq,
                                          const int32_t* __restrict__ depth, const int32_t* __restrict__ seq_len,
                                          const int32_t* __restrict__ row_off, int B, T* __restrict__ q_out,
                                          T* __restrict__ k_slab, T* __restrict__ v_slab, int H, int Hkv, int D, int max_seq,
@@ -399,11 +409,7 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_kv_write_vec_kernel(const P
     float sn[4], cs[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        // angle in fp64 (positions reach thousands of radians), reduced to [-pi, pi] there; sin/cos of the reduced
-        // angle in fp32 are then accurate to ~1e-7
-        const double ang = (double)pos * inv_freq[i + e];
-        const double red = ang - 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
-        sincosf((float)red, &sn[e], &cs[e]);
+        rotation((double)pos * inv_freq[i + e], sn[e], cs[e]);
     }
     pdl_wait();
     TRJ_TL_BEGIN(TRJ_TL_ROPE);
@@ -443,6 +449,57 @@ __global__ void __launch_bounds__(ROPE_THREADS) rope_kv_write_vec_kernel(const P
         store_split4<T>(v_slab, nullptr, cache_at, acc[4]);
         store_split4<T>(v_slab, nullptr, cache_at + half, acc[5]);
     }
+    TRJ_TL_END(TRJ_TL_ROPE);                                 // thread 0's own stores; the others' end within the same few hundred ns
+}
+
+// The same with the rows' table: heads are those of the projection result, H of q, Hkv of k, Hkv of v (only moved).
+template <typename T, int BATCH>            // BATCH: split-K pieces requested at a time
+__global__ void __launch_bounds__(ROPE_THREADS) rope_kv_write_kernel(const Parts qkv, const float* __restrict__ rot, const int2* __restrict__ row_at,
+                                         T* __restrict__ q_out, T* __restrict__ k_slab, T* __restrict__ v_slab, int H, int Hkv, int D, int max_seq) {
+    pdl_launch_dependents();
+    const int half = D >> 1, per_head = half >> 2, heads = H + 2 * Hkv;
+    const int row = blockIdx.x, hh = (int)(blockIdx.y * ROPE_THREADS + threadIdx.x) / per_head;
+    const int i = ((int)threadIdx.x % per_head) * 4;
+    TRJ_TL_DECL;
+    if (hh >= heads) return;                                 // never thread 0: a CTA's first thread has a head
+    const float* src = qkv.ptr + ((size_t)row * heads + hh) * D + i;
+    pdl_wait();
+    TRJ_TL_BEGIN(TRJ_TL_ROPE);
+    const float4 cs = *reinterpret_cast<const float4*>(rot + (size_t)row * D + i), sn = *reinterpret_cast<const float4*>(rot + (size_t)row * D + half + i);
+    const int2 at = row_at[row];
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+    for (int s0 = 0; s0 < qkv.splits; s0 += BATCH) {         // added in ascending order
+        float4 a[BATCH], b[BATCH];
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j)
+            if (s0 + j < qkv.splits) {
+                const float* piece = src + (size_t)(s0 + j) * qkv.stride;
+                a[j] = *reinterpret_cast<const float4*>(piece);
+                b[j] = *reinterpret_cast<const float4*>(piece + half);
+            }
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j)
+            if (s0 + j < qkv.splits) {
+                lo.x += a[j].x; lo.y += a[j].y; lo.z += a[j].z; lo.w += a[j].w;
+                hi.x += b[j].x; hi.y += b[j].y; hi.z += b[j].z; hi.w += b[j].w;
+            }
+    }
+    if (hh < H + Hkv) {
+        const float4 l = lo, h = hi;
+        lo = make_float4(l.x * cs.x - h.x * sn.x, l.y * cs.y - h.y * sn.y, l.z * cs.z - h.z * sn.z, l.w * cs.w - h.w * sn.w);
+        hi = make_float4(h.x * cs.x + l.x * sn.x, h.y * cs.y + l.y * sn.y, h.z * cs.z + l.z * sn.z, h.w * cs.w + l.w * sn.w);
+    }
+    T* dst;
+    size_t to;
+    if (hh < H) {
+        dst = q_out; to = ((size_t)row * H + hh) * D + i;
+    } else {
+        dst = hh < H + Hkv ? k_slab : v_slab;
+        to = (((size_t)at.x * Hkv + (hh < H + Hkv ? hh - H : hh - H - Hkv)) * max_seq + at.y) * D + i;
+        if (!TRJ_DEBUG_CHECK((unsigned)at.y < (unsigned)max_seq, DBG_ROPE_ROW)) return;
+    }
+    store_split4<T>(dst, nullptr, to, lo);
+    store_split4<T>(dst, nullptr, to + half, hi);
     TRJ_TL_END(TRJ_TL_ROPE);                                 // thread 0's own stores; the others' end within the same few hundred ns
 }
 
@@ -558,18 +615,40 @@ __global__ void swiglu_kernel(const Parts gu, T* __restrict__ act, T* __restrict
 }
 
 // Four columns per thread (f a multiple of 4).
+__device__ __forceinline__ float4 silu_mul(const float4& g, const float4& u) {
+    return make_float4(g.x / (1.f + expf(-g.x)) * u.x, g.y / (1.f + expf(-g.y)) * u.y,
+                       g.z / (1.f + expf(-g.z)) * u.z, g.w / (1.f + expf(-g.w)) * u.w);
+}
+// From split-K pieces.  64 registers, eight CTAs an SM: with 101 the 710 CTAs of a 33-row step take two waves (3.22 against
+// 3.14 ms a step), with 51 or 42 the eight loads of an item no longer fit and go one after the other (3.19, 3.26 ms).
+constexpr int SWIGLU_THREADS = 128, SWIGLU_MAX_CTAS = 2368;
 template <typename T>
-__global__ void swiglu_vec_kernel(const Parts gu, T* __restrict__ act, T* __restrict__ act_lo, int rows, int f) {
+__global__ void __launch_bounds__(SWIGLU_THREADS, 8) swiglu_pieces_kernel(const Parts gu, T* __restrict__ act, T* __restrict__ act_lo, int rows, int f) {
     pdl_prologue();
     TRJ_TL_DECL; TRJ_TL_BEGIN(TRJ_TL_SWIGLU);
     const int f4 = f >> 2;
     const size_t n4 = (size_t)rows * f4;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         const size_t r = i / f4, c4 = i % f4;
-        const float4 g = parts_at4_batched(gu, r * 2 * f4 + c4), u = parts_at4_batched(gu, r * 2 * f4 + f4 + c4);
-        store_split4<T>(act, act_lo, 4 * i,
-                        make_float4(g.x / (1.f + expf(-g.x)) * u.x, g.y / (1.f + expf(-g.y)) * u.y,
-                                    g.z / (1.f + expf(-g.z)) * u.z, g.w / (1.f + expf(-g.w)) * u.w));
+        store_split4<T>(act, act_lo, 4 * i, silu_mul(parts_at4_batched<4>(gu, r * 2 * f4 + c4), parts_at4_batched<4>(gu, r * 2 * f4 + f4 + c4)));
+    }
+#ifdef TRJ_TIMELINE
+    __syncthreads();
+#endif
+    TRJ_TL_END(TRJ_TL_SWIGLU);
+}
+// From finished sums (many rows): blockIdx.y walks the rows instead of a 64-bit division per item, and without the pieces'
+// buffers 16 CTAs fit an SM.  1024 rows x 11008 (135 MB): 47 -> 29 us.
+template <typename T>
+__global__ void __launch_bounds__(SWIGLU_THREADS) swiglu_rows_kernel(const float4* __restrict__ gu, T* __restrict__ act, T* __restrict__ act_lo, int rows, int f) {
+    pdl_prologue();
+    TRJ_TL_DECL; TRJ_TL_BEGIN(TRJ_TL_SWIGLU);
+    const int f4 = f >> 2, c4 = blockIdx.x * SWIGLU_THREADS + threadIdx.x;
+    if (c4 < f4) {
+        for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+            const size_t at = (size_t)r * 2 * f4 + c4;
+            store_split4<T>(act, act_lo, (size_t)r * f + 4 * c4, silu_mul(gu[at], gu[at + f4]));
+        }
     }
 #ifdef TRJ_TIMELINE
     __syncthreads();
@@ -1105,11 +1184,12 @@ uint64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); 
     if ((dtype) == TRJ_BF16) { using T = __nv_bfloat16; __VA_ARGS__; } \
     else { using T = float; __VA_ARGS__; }
 
-cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens, float* h,
-                         int32_t rows, int32_t d, cudaStream_t st) {
+cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens, float* h, int32_t d, const double* inv_freq, int32_t D,
+                         const int32_t* depth, const Batch& bt, const Rotary& rot, cudaStream_t st) {
     count_launch();
     cudaError_t launch_err = cudaSuccess;
-    DISPATCH_T(dtype, launch_err = launch_chain(embed_kernel<T>, dim3(rows), dim3(256), 0, st, (const T*)embed, tokens, h, d));
+    DISPATCH_T(dtype, launch_err = launch_chain(embed_kernel<T>, dim3(bt.rows_total), dim3(256), 0, st, (const T*)embed, tokens, h, d, inv_freq, D / 2,
+                                                depth, bt.seq_len, bt.row_off, bt.B, rotary_table_used(bt.rows_total) ? rot.table : nullptr, rot.row_at));
     return launch_err != cudaSuccess ? launch_err : cudaGetLastError();
 }
 
@@ -1117,10 +1197,14 @@ cudaError_t launch_add_rmsnorm(float* h, const Parts& add, const float* gain, vo
                                int32_t rows, int32_t d, float eps, cudaStream_t st) {
     count_launch();
     cudaError_t launch_err = cudaSuccess;
-    const bool vec = d % 4 == 0 && d <= 4 * RMS_THREADS * RMS_CHUNKS && add.stride % 4 == 0 &&
+    const bool vec = d % 4 == 0 && d <= RMS_MAX_D && add.stride % 4 == 0 &&
                      ((uintptr_t)h | (uintptr_t)add.ptr | (uintptr_t)gain | (uintptr_t)x | (uintptr_t)x_lo) % 16 == 0;
     if (vec) {
-        DISPATCH_T(dtype, launch_err = launch_chain(add_rmsnorm_vec_kernel<T>, dim3(rows), dim3(RMS_THREADS), 0, st, h, add, gain, (T*)x, (T*)x_lo, d, eps));
+#define RMS(THREADS, CHUNKS) \
+    DISPATCH_T(dtype, launch_err = launch_chain(add_rmsnorm_vec_kernel<T, THREADS, CHUNKS>, dim3(rows), dim3(THREADS), 0, st, h, add, gain, (T*)x, (T*)x_lo, d, eps))
+        if (rows <= RMS_FEW_ROWS) { RMS(RMS_FEW_ROWS_THREADS, 2); }
+        else { if (d <= 4096) { RMS(256, 4); } else { RMS(256, 8); } }
+#undef RMS
     } else {
         DISPATCH_T(dtype, launch_err = launch_chain(add_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, h, add, gain, (T*)x, (T*)x_lo, d, eps));
     }
@@ -1154,22 +1238,24 @@ cudaError_t launch_gemm_simt(const void* x, const void* x_lo, const void* w, flo
     return cudaGetLastError();
 }
 
-cudaError_t launch_rope_kv_write(const Parts& qkv, const double* inv_freq, const int32_t* depth,
-                                 const Batch& bt, void* q_out, void* k_slab, void* v_slab, int32_t dtype,
-                                 int32_t H, int32_t Hkv, int32_t D, int32_t max_seq, cudaStream_t st) {
+bool rotary_table_used(int32_t rows) { return rows > ROPE_FEW_ROWS; }
+
+cudaError_t launch_rope_kv_write(const Parts& qkv, const Rotary& rot, const double* inv_freq, const int32_t* depth, const Batch& bt, void* q_out,
+                                 void* k_slab, void* v_slab, int32_t dtype, int32_t H, int32_t Hkv, int32_t D, int32_t max_seq, cudaStream_t st) {
+    if (D % 8 != 0 || ROPE_THREADS % (D / 8) != 0 || qkv.stride % 4 != 0 || ((uintptr_t)qkv.ptr % 16) != 0) return cudaErrorInvalidValue;
     count_launch();
+    const int per_head = D / 8;                              // threads per head
     cudaError_t launch_err = cudaSuccess;
-    const int per_head = D / 8;                              // threads per head in the vector kernel
-    const int hpc = per_head > 0 ? std::max(1, std::min(H, ROPE_THREADS / per_head)) : 1;
-    const bool vec = D % 8 == 0 && per_head <= ROPE_THREADS && qkv.stride % 4 == 0 && ((uintptr_t)qkv.ptr % 16) == 0;
-    if (vec) {
-        dim3 grid(bt.rows_total, (H + hpc - 1) / hpc);
-        DISPATCH_T(dtype, launch_err = launch_chain(rope_kv_write_vec_kernel<T>, grid, dim3(per_head * hpc), 0, st, qkv, inv_freq, depth,
-                                                    bt.seq_len, bt.row_off, bt.B, (T*)q_out, (T*)k_slab, (T*)v_slab, H, Hkv, D, max_seq, hpc));
+    if (rotary_table_used(bt.rows_total)) {
+        const int heads_per_cta = ROPE_THREADS / per_head;
+        DISPATCH_T(dtype, launch_err = launch_chain(qkv.splits > 1 ? rope_kv_write_kernel<T, 4> : rope_kv_write_kernel<T, 1>,
+                                                    dim3(bt.rows_total, (H + 2 * Hkv + heads_per_cta - 1) / heads_per_cta), dim3(ROPE_THREADS), 0, st,
+                                                    qkv, rot.table, rot.row_at, (T*)q_out, (T*)k_slab, (T*)v_slab, H, Hkv, D, max_seq));
     } else {
-        dim3 grid(bt.rows_total, H);
-        DISPATCH_T(dtype, launch_err = launch_chain(rope_kv_write_kernel<T>, grid, dim3(64), 0, st, qkv, inv_freq, depth, bt.seq_len, bt.row_off,
-                                                    bt.B, (T*)q_out, (T*)k_slab, (T*)v_slab, H, Hkv, D, max_seq));
+        const int hpc = std::max(1, std::min(H, ROPE_THREADS / per_head));
+        DISPATCH_T(dtype, launch_err = launch_chain(rope_kv_write_few_kernel<T>, dim3(bt.rows_total, (H + hpc - 1) / hpc), dim3(per_head * hpc), 0, st,
+                                                    qkv, inv_freq, depth, bt.seq_len, bt.row_off, bt.B, (T*)q_out, (T*)k_slab, (T*)v_slab, H, Hkv, D,
+                                                    max_seq, hpc));
     }
     return launch_err != cudaSuccess ? launch_err : cudaGetLastError();
 }
@@ -1198,9 +1284,13 @@ cudaError_t launch_swiglu(const Parts& gu, void* act, void* act_lo, int32_t dtyp
     cudaError_t launch_err = cudaSuccess;
     const bool vec = f % 4 == 0 && gu.stride % 4 == 0 && ((uintptr_t)gu.ptr % 16) == 0;
     const size_t n = (size_t)rows * (vec ? f / 4 : f);
-    const int blocks = (int)((n + 127) / 128 < 2368 ? (n + 127) / 128 : 2368);
-    if (vec) {
-        DISPATCH_T(dtype, launch_err = launch_chain(swiglu_vec_kernel<T>, dim3(blocks), dim3(128), 0, st, gu, (T*)act, (T*)act_lo, rows, f));
+    const int blocks = (int)std::min<size_t>((n + SWIGLU_THREADS - 1) / SWIGLU_THREADS, SWIGLU_MAX_CTAS);
+    if (vec && gu.splits > 1) {
+        DISPATCH_T(dtype, launch_err = launch_chain(swiglu_pieces_kernel<T>, dim3(blocks), dim3(SWIGLU_THREADS), 0, st, gu, (T*)act, (T*)act_lo, rows, f));
+    } else if (vec) {
+        const int across = (f / 4 + SWIGLU_THREADS - 1) / SWIGLU_THREADS;
+        DISPATCH_T(dtype, launch_err = launch_chain(swiglu_rows_kernel<T>, dim3(across, std::min(rows, std::max(1, SWIGLU_MAX_CTAS / across))),
+                                                    dim3(SWIGLU_THREADS), 0, st, (const float4*)gu.ptr, (T*)act, (T*)act_lo, rows, f));
     } else {
         DISPATCH_T(dtype, launch_err = launch_chain(swiglu_kernel<T>, dim3(blocks), dim3(128), 0, st, gu, (T*)act, (T*)act_lo, rows, f));
     }

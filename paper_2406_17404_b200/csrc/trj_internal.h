@@ -120,8 +120,13 @@ struct TopTable { TopEntry* entries; int32_t store_y; };
 bool gemm_top_table_ok(int32_t M, int32_t N, int32_t K, int32_t dtype, bool pair);
 inline size_t gemm_top_table_entries(int32_t rows, int32_t N) { return (size_t)rows * ((N + 127) / 128) * 4; }
 
-cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens, float* h,
-                         int32_t rows, int32_t d, cudaStream_t st);
+// What every layer's rotary step needs of a row of the forward, worked out by the embedding kernel: cosines then sines of its
+// position, [rows][head_dim], and (sequence, cache row) of its K/V.
+struct Rotary { float* table; int2* row_at; };
+bool rotary_table_used(int32_t rows);       // few rows work their rotations out themselves, ahead of their wait
+// h = embedding rows of `tokens`; fills `rot` for the rows of bt (position seq_len[b] + depth[row]).
+cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens, float* h, int32_t d, const double* inv_freq, int32_t D,
+                         const int32_t* depth, const Batch& bt, const Rotary& rot, cudaStream_t st);
 // h += add (when add != nullptr, h is updated in place); x = rmsnorm(h) * gain, stored as dtype.
 // In bf16 models x is written as a bf16 pair: x (hi) and x_lo (the rounding error of hi); x_lo may be null.
 cudaError_t launch_add_rmsnorm(float* h, const Parts& add, const float* gain, void* x, void* x_lo, int32_t dtype,
@@ -150,12 +155,11 @@ cudaError_t launch_gemm(const void* x, const void* x_lo, const void* w, float* y
                         int32_t dtype, void* workspace, size_t workspace_bytes, cudaStream_t st, Parts* parts = nullptr,
                         const WeightPrefetch* ahead = nullptr, int* status = nullptr, const TopTable* top = nullptr);
 
-// Rotary embedding of q and k at position seq_len[b] + depth[row]; q -> q_out [rows][H][D];
-// k, v -> cache rows seq_len[b] + local row of the layer slab [B][Hkv][max_seq][D].  The projection result has
-// (H + 2 * Hkv) * D values per row: H query heads, then Hkv key heads, then Hkv value heads.
-cudaError_t launch_rope_kv_write(const Parts& qkv, const double* inv_freq, const int32_t* depth,
-                                 const Batch& bt, void* q_out, void* k_slab, void* v_slab, int32_t dtype,
-                                 int32_t H, int32_t Hkv, int32_t D, int32_t max_seq, cudaStream_t st);
+// Rotary embedding of q and k at position seq_len[b] + depth[row]; q -> q_out [rows][H][D]; k, v -> cache rows seq_len[b] + local row of the layer slab
+// [B][Hkv][max_seq][D].  The projection result has (H + 2 * Hkv) * D values per row: H query heads, then Hkv key heads, then
+// Hkv value heads.
+cudaError_t launch_rope_kv_write(const Parts& qkv, const Rotary& rot, const double* inv_freq, const int32_t* depth, const Batch& bt, void* q_out,
+                                 void* k_slab, void* v_slab, int32_t dtype, int32_t H, int32_t Hkv, int32_t D, int32_t max_seq, cudaStream_t st);
 // Attention: H query heads over Hkv K/V heads (query head h reads K/V head h / (H / Hkv)).
 cudaError_t launch_tree_attention_generic(const void* q, const void* k_slab, const void* v_slab,
                                           const uint64_t* anc, int32_t anc_words, const Batch& bt,

@@ -1,0 +1,39 @@
+"""Element-wise kernels on either side of the row counts where their form changes (one row per SM), through a decoder."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+from gpu_util import i32
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype,heads", [("f32", 4), ("bf16", 2)])
+@pytest.mark.parametrize("rows", [148, 149, 300])
+def test_prompt_cache_rows_and_first_token(trj, dtype, heads, rows):
+    """A prompt of `rows` tokens is one forward of that many rows: every layer's K/V rows (rotary table, RMSNorm and SwiGLU of
+    many rows) and the greedy token against the oracle."""
+    from dataclasses import replace
+    from paper_2406_17404_b200.decode import upload_weights
+    cfg = replace(synth.TINY, dtype=dtype, n_kv_heads=heads)
+    layers = [synth.layer_weights(cfg, 3, l) for l in range(cfg.n_layers)]
+    glob = synth.global_weights(cfg, 3)
+    model = trj.Model(cfg, *upload_weights(cfg, layers, glob), max_batch=1, max_seq=512, max_rows=128)
+    f64 = lambda d: {k: np.asarray(v, np.float64) for k, v in d.items()}
+    dec = oracle.Decoder(cfg, [f64(l) for l in layers], f64(glob))
+    prompt = synth.prompt(rows, rows, cfg.vocab)
+    first = int(model.prefill(i32(prompt)).item())
+    cache = dec.new_cache(512)
+    want = dec.forward_rows(cache, prompt, synth.chain_parents(rows))
+    k, v = (c[:, 0, :, :rows].float().cpu().numpy() for c in (model.k_cache, model.v_cache))
+    # bf16: q and K/V roundings that fall the other way (2^-8 relative each) reach the next layer as input errors of that size
+    # times its O(0.3) values, then each value is rounded itself: one bf16 step (2^-7) of the value, or of 0.25 below that;
+    # fp32: sums of 256 and 688 products
+    for got, ref in ((k, cache.k), (v, cache.v)):
+        ref = np.asarray(ref)[:, :, :rows]
+        tol = np.maximum(np.abs(ref), 0.25) * 2.0 ** -7 if dtype == "bf16" else 2e-5
+        assert (np.abs(got - ref) <= tol).all()
+    margin = oracle.top2_margin(np.asarray(want)[-1:])[0]
+    assert margin < 1e-2 or first == int(oracle.node_argmax(np.asarray(want)[-1:])[0])
