@@ -87,6 +87,7 @@ extern "C" trj_status trj_argmax_accept(const void* logits, int32_t dtype, int32
     TRJ_REQUIRE(rows_total <= B * TRJ_MAX_ROWS, TRJ_ECAPACITY, "argmax_accept: too many rows");
     TRJ_REQUIRE(workspace && aligned(workspace, 256) && workspace_bytes >= argmax_workspace_bytes(rows_total, B),
                 TRJ_ECAPACITY, "argmax_accept: workspace too small or misaligned");
+    ChainScope chain;                        // these kernels wait for their predecessor before reading anything
     TRJ_CHECK_CUDA(launch_topk_accept(logits, dtype, V, 1, tokens, parent, depth, row_off, B, rows_total, nullptr, node_argmax,
                                       margin, k_acc, path, bonus, true, workspace, (cudaStream_t)stream));
     return TRJ_OK;
@@ -109,6 +110,7 @@ extern "C" trj_status trj_topk_accept(const void* logits, int32_t dtype, int32_t
     TRJ_REQUIRE(rows_total <= B * TRJ_MAX_ROWS, TRJ_ECAPACITY, "topk_accept: too many rows");
     TRJ_REQUIRE(workspace && aligned(workspace, 256) && workspace_bytes >= topk_workspace_bytes(),
                 TRJ_ECAPACITY, "topk_accept: workspace too small or misaligned");
+    ChainScope chain;                        // these kernels wait for their predecessor before reading anything
     TRJ_CHECK_CUDA(launch_topk_accept(logits, dtype, V, K, tokens, parent, depth, row_off, B, rows_total, topk, node_argmax,
                                       margin, k_acc, path, bonus, true, workspace, (cudaStream_t)stream));
     return TRJ_OK;
@@ -146,6 +148,7 @@ extern "C" trj_status trj_compact_rows(void* k_cache, void* v_cache, int32_t L, 
     TRJ_REQUIRE(B <= TRJ_MAX_BATCH, TRJ_ECAPACITY, "compact_rows: batch %d exceeds %d", B, TRJ_MAX_BATCH);
     TRJ_REQUIRE((D * dtype_size(dtype)) % 16 == 0 && aligned(k_cache, 16) && aligned(v_cache, 16), TRJ_EINVAL,
                 "compact_rows: cache rows must be multiples of 16 bytes and 16-byte aligned");
+    ChainScope chain;                        // these kernels wait for their predecessor before reading anything
     TRJ_CHECK_CUDA(launch_compact(k_cache, v_cache, L, B, B, H, max_seq, D, dtype, seq_len, k_acc, path,
                                   (cudaStream_t)stream));
     return TRJ_OK;

@@ -1,19 +1,26 @@
 // Tree-masked attention for sm_100a (bf16, head_dim 128, up to 128 tree rows per sequence).
 //
-// Work is cut into units of one 128-key tile of one (sequence, head); the units, laid out sequence-
-// major, are dealt in equal contiguous ranges to a persistent grid of one CTA per SM, so a long prefix
-// is split over several CTAs (split-KV) and short sequences are packed several per CTA.  Inside a CTA:
-//   * one thread streams Q (per segment) and the K/V tiles with TMA into 128-byte-swizzled shared memory;
-//   * one thread issues tcgen05.mma: S = Q.K^T into TMEM (two S buffers), then O += P.V with P read from
-//     TMEM as well (two P buffers) and the accumulator resident in TMEM for the whole segment;
-//   * eight (or sixteen) warps do the softmax: a thread owns half (a quarter) of one query row (TMEM lane = row, 64 of the 128
-//     columns); they read S once into registers, apply the ancestor bitmask on tiles that reach the tree
-//     rows, keep an online softmax whose running maximum is only raised when a tile exceeds it by more
-//     than 2^8 (then O is rescaled in TMEM), and store P as bf16 pairs back into TMEM, where the second
-//     MMA reads it as its A operand: the softmax of a tile never waits for the previous tile's P.V.
-// A segment that covers all tiles of its (sequence, head) writes the normalised bf16 output itself;
-// otherwise it leaves (max, sum, O) in the workspace and a second kernel merges the pieces in a fixed
-// order.  Every wait on an mbarrier is bounded; on expiry the CTA records TRJ_ETIMEOUT and leaves.
+// Work is cut into units of one 128-key tile of one (sequence, head).  A CTA works on TWO STREAMS of units at a time: what
+// bounds a stream is its chain of dependent steps (scores -> softmax -> P.V -> next scores: 2.3 us a tile with a bf16 P and
+// 4.6 us with a pair in the one-stream form of this kernel, against 1.4 us that the tile's 64 KB take from HBM and 0.6 us
+// of exponentials), so the chains of two streams are interleaved.  Inside a CTA:
+//   * one thread per stream brings Q (per segment) and the K/V tiles with TMA into 128-byte-swizzled shared memory: a slot for
+//     K, free again once the scores of its tile are complete, and one for V, free once P.V is (a barrier that two
+//     consumers wait on by parity must not be shared between the streams: one could be a phase ahead of the other);
+//   * one thread per stream issues tcgen05.mma: S = Q.K^T into the stream's score buffer in TMEM, then O += P.V with P read
+//     from that same buffer and the accumulator resident in TMEM for the whole segment (one thread for both streams was the
+//     bottleneck: 2200 cycles a tile, most of them the latency of its waits);
+//   * eight warps per stream do the softmax: they read S once into registers, apply the ancestor bitmask on tiles that
+//     reach the tree rows, keep an online softmax whose running maximum is only raised when a tile exceeds it by more
+//     than 2^8 (then O is rescaled in TMEM), and store P as bf16 over the scores it comes from, where the second MMA reads it
+//     as its A operand.
+// Up to 64 tree rows (kernel of 64-row streams): stream 0 is the lower, stream 1 the upper half of the 128 TMEM lanes; each
+// MMA computes all 128 lanes and the other stream's half is not looked at.  Four threads share a row, so a tree of up to 64
+// rows keeps all four quarters of the SM busy.  More rows: both streams use all lanes, two threads share a row.
+// A segment (a stream's consecutive units of one (sequence, head)) that covers all tiles of its (sequence, head) writes the
+// normalised bf16 output itself.  Otherwise, one sequence: the head's pieces lie in the shared memory of a cluster and are
+// merged there; a batch: (max, sum, O) goes to the workspace and a second kernel merges the pieces in a fixed order.
+// Every wait on an mbarrier is bounded; on expiry the CTA records TRJ_ETIMEOUT and leaves.
 #include <cuda.h>
 #include <cstdlib>
 #include <mutex>
@@ -24,24 +31,25 @@
 namespace trj {
 namespace {
 
-constexpr int AT_ROWS = 128;                 // query rows per CTA = UMMA M = TMEM lanes
+constexpr int AT_LANES = 128;                // UMMA M = TMEM lanes
 constexpr int AT_KEYS = 128;                 // keys per tile
 constexpr int AT_D = 128;                    // head_dim
-// The softmax is done by 4 * SPLIT warps: SPLIT threads share a query row, each taking a column group of a tile
-// (template parameter of the kernel: 2 for one sequence with full row groups, 4 for batches of small trees, where
-// half of the row groups are empty and more threads per row pay off).
-__host__ __device__ constexpr int at_threads(int split) { return 32 * 4 * split + 64; }   // softmax warps + TMA warp + MMA warp
+constexpr int AT_STREAMS = 2;
+constexpr int AT_STREAM_WARPS = 8, AT_SM_WARPS = AT_STREAMS * AT_STREAM_WARPS;      // softmax warps
+constexpr int AT_W_COPY = AT_SM_WARPS, AT_W_MMA = AT_SM_WARPS + AT_STREAMS;      // a TMA warp and an MMA warp per stream
+constexpr int AT_THREADS = 32 * (AT_SM_WARPS + 2 * AT_STREAMS);
 constexpr uint32_t AT_SUB = 128 * 128;       // one [128 x 64 bf16] swizzled sub-tile: 16 KB
-constexpr uint32_t AT_TILE = 2 * AT_SUB;     // Q, P, a K tile or a V tile: 32 KB
-constexpr int AT_RING = 5;                   // K/V ring slots; load n = 2g + (0: K, 1: V) of tile g goes to slot n % 5
-constexpr uint32_t AT_SMEM = (1 + AT_RING) * AT_TILE + 1024;
+constexpr uint32_t AT_TILE = 2 * AT_SUB;     // a K tile, a V tile, 128 rows of Q: 32 KB
+// Q (64-row streams: one tile, a half each; wide: a tile each), then a K slot and a V slot per stream
+__host__ __device__ constexpr int at_q_tiles(bool wide) { return wide ? 2 : 1; }
+__host__ __device__ constexpr uint32_t at_smem(bool wide) { return (uint32_t)(at_q_tiles(wide) + 2 * AT_STREAMS) * AT_TILE + 1024; }
 constexpr float AT_RESCALE_GAP = 8.f;        // raise the running max only when exceeded by 2^8
-constexpr int AT_PIECE_STRIDE = AT_D + 4;      // floats per row of a piece in shared memory (16-byte stores without bank conflicts)
-constexpr size_t AT_SLOT_FLOATS = (size_t)AT_D * AT_ROWS + 2 * AT_ROWS;   // O^T [d][row], m[row], l[row]
+constexpr size_t AT_SLOT_FLOATS = (size_t)AT_D * AT_LANES + 2 * AT_LANES;   // O^T [d][row], m[row], l[row]
 
-// barrier indices
-enum { B_KV_FULL = 0, B_KV_EMPTY = 5, B_Q_FULL = 10, B_Q_EMPTY = 11, B_S_FULL = 12, B_P_READY = 14, B_P_FREE = 16,
-       B_O_READY = 18, B_O_FREE = 19, B_COUNT = 20 };
+// barrier indices, one barrier per stream each; the last two: every CTA of the cluster has reached the merge; the other CTAs'
+// pieces have arrived
+enum { B_K_FULL = 0, B_K_EMPTY = 2, B_V_FULL = 4, B_V_EMPTY = 6, B_Q_FULL = 8, B_Q_EMPTY = 10, B_S_FULL = 12, B_P_READY = 14, B_O_READY = 16,
+       B_O_FREE = 18, B_PEERS = 20, B_RECEIVED = 21, B_COUNT = 22 };
 
 struct AtParams {
     const int32_t* seq_len; const int32_t* row_off; const uint64_t* anc;
@@ -52,8 +60,11 @@ struct AtParams {
     float* slots;                // partial results, AT_SLOT_FLOATS each
     int* status;
     float scale_log2;            // log2(e) / sqrt(D)
-    int cluster;                 // CTAs per thread-block cluster that share one head (1: no clusters)
+    int cluster;                 // one sequence: CTAs per thread-block cluster that share one head; 0: a batch
+    int in_chain;                // the batch geometry and the ancestor masks are older than the chain: they may be read before the wait
     int early_ok;                // cache rows below seq_len are older than the chain: they may be fetched before the wait
+    int rows_cap;                // most rows of a tree that the launched kernel takes
+    int streams;                 // of the whole launch (batches; see build_range)
     int shared_cache;            // every sequence of the batch uses the cache of sequence 0 (pieces of one prompt chunk)
 };
 
@@ -83,17 +94,18 @@ __device__ __forceinline__ void umma8_qk(uint32_t tmem_d, uint32_t a_lo, uint32_
                  ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc) : "memory");
 }
 #undef TRJ_MMA_SS
-// O (+)= P.V for one tile: P from tensor memory (16 keys = 8 columns per step), V MN-major (16 keys = 2048 bytes per step).
-#define TRJ_MMA_TS(kk, pred)                                                              \
-    "add.u32 ta, %1, " #kk "*8;\n\tadd.u32 bl, %2, " #kk "*128;\n\t"                      \
+// O (+)= P.V for one tile: P from tensor memory (16 keys = 8 columns per step; every 32 keys' P lies in the first columns of
+// the 32 score columns it replaces), V MN-major (16 keys = 2048 bytes per step).
+#define TRJ_MMA_TS(col, kk, pred)                                                         \
+    "add.u32 ta, %1, " #col ";\n\tadd.u32 bl, %2, " #kk "*128;\n\t"                      \
     "mov.b64 db, {bl, %3};\n\t"                                                            \
     "tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %4, " #pred ";\n\t"
 __device__ __forceinline__ void umma8_pv(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
                                          uint32_t accumulate_first) {
     asm volatile("{\n\t.reg .pred pt, pf;\n\t.reg .b32 ta, bl;\n\t.reg .b64 db;\n\t"
                  "setp.eq.b32 pt, 0, 0;\n\tsetp.ne.b32 pf, %5, 0;\n\t"
-                 TRJ_MMA_TS(0, pf) TRJ_MMA_TS(1, pt) TRJ_MMA_TS(2, pt) TRJ_MMA_TS(3, pt)
-                 TRJ_MMA_TS(4, pt) TRJ_MMA_TS(5, pt) TRJ_MMA_TS(6, pt) TRJ_MMA_TS(7, pt)
+                 TRJ_MMA_TS(0, 0, pf) TRJ_MMA_TS(8, 1, pt) TRJ_MMA_TS(32, 2, pt) TRJ_MMA_TS(40, 3, pt)
+                 TRJ_MMA_TS(64, 4, pt) TRJ_MMA_TS(72, 5, pt) TRJ_MMA_TS(96, 6, pt) TRJ_MMA_TS(104, 7, pt)
                  "}"
                  ::"r"(tmem_d), "r"(tmem_a), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate_first) : "memory");
 }
@@ -112,63 +124,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
-// Two back-to-back 32-column loads with one wait (64 consecutive columns).
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
-    uint32_t r[64];
-#define TRJ_LD32(base, off)                                                                                          \
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "                                                           \
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "                            \
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"            \
-                 : "=r"(r[off + 0]), "=r"(r[off + 1]), "=r"(r[off + 2]), "=r"(r[off + 3]), "=r"(r[off + 4]), "=r"(r[off + 5]),   \
-                   "=r"(r[off + 6]), "=r"(r[off + 7]), "=r"(r[off + 8]), "=r"(r[off + 9]), "=r"(r[off + 10]), "=r"(r[off + 11]), \
-                   "=r"(r[off + 12]), "=r"(r[off + 13]), "=r"(r[off + 14]), "=r"(r[off + 15]), "=r"(r[off + 16]),               \
-                   "=r"(r[off + 17]), "=r"(r[off + 18]), "=r"(r[off + 19]), "=r"(r[off + 20]), "=r"(r[off + 21]),               \
-                   "=r"(r[off + 22]), "=r"(r[off + 23]), "=r"(r[off + 24]), "=r"(r[off + 25]), "=r"(r[off + 26]),               \
-                   "=r"(r[off + 27]), "=r"(r[off + 28]), "=r"(r[off + 29]), "=r"(r[off + 30]), "=r"(r[off + 31])                \
-                 : "r"(base) : "memory")
-    TRJ_LD32(taddr, 0);
-    TRJ_LD32(taddr + 32, 32);
-#undef TRJ_LD32
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-                 "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-                 ::"r"(taddr),
-                   "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-                   "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-                   "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-                   "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15])),
-                   "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])), "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])),
-                   "r"(__float_as_uint(v[20])), "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-                   "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])), "r"(__float_as_uint(v[27])),
-                   "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])), "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-                 : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_st32u(uint32_t taddr, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-                 "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-                 ::"r"(taddr),
-                   "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-                   "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-                   "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
-                   "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-                 : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tmem_st16u(uint32_t taddr, const uint32_t* v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
                  "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
                  ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-                 : "memory");
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                 : "memory");                                // no wait: pair with tmem_wait_st
 }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);      // .x (low half) = a
     return *reinterpret_cast<const uint32_t*>(&h);
@@ -197,17 +160,6 @@ __device__ __forceinline__ void store4_split(__nv_bfloat16* hi, __nv_bfloat16* l
         *reinterpret_cast<uint2*>(lo) = make_uint2(pack_bf16(a - bf16_round(a), b - bf16_round(b)),
                                                    pack_bf16(c - bf16_round(c), d - bf16_round(d)));
 }
-// Loads from distributed shared memory.
-__device__ __forceinline__ float ld_cluster(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
-}
 // 128-bit (lo, hi) shifts by 0..127 bits; the left shift fills the vacated low bits with ones.
 __device__ __forceinline__ void shr128(uint64_t& lo, uint64_t& hi, int n) {
     if (n == 0) return;
@@ -229,241 +181,284 @@ struct Sched {
     int S[TRJ_MAX_BATCH];               // cached rows of each sequence (a copy of seq_len: no global load on the critical path)
     int row0[TRJ_MAX_BATCH + 1];        // a copy of row_off
     int first[TRJ_MAX_BATCH + 1];       // first unit of each sequence (the launcher checks that the count fits an int)
-    int u_begin, u_end;                 // this CTA's units
-    __device__ void locate(int u, Where& w) const {
+    int head;                           // one sequence: the head of this CTA's cluster; -1 for a batch
+    int whole;                          // batches: every stream takes at most one (sequence, head), whole
+    int u_begin[AT_STREAMS], u_end[AT_STREAMS];      // this CTA's units
+    __device__ int rows(int b, int cap) const { return min(max(row0[b + 1] - row0[b], 0), cap); }
+    __device__ void locate(int u, Where& w, int cap) const {
         int b = 0;
         while (b + 1 < B && u >= first[b + 1]) ++b;
         const int r = u - first[b];
         w.b = b; w.tiles = tiles[b];
-        w.h = r / w.tiles; w.t = r % w.tiles;
-        w.S = S[b]; w.rows = row0[b + 1] - row0[b];
+        w.h = head >= 0 ? head : r / w.tiles;
+        w.t = r - w.h * w.tiles;
+        w.S = S[b]; w.rows = rows(b, cap);
         w.bh = b * H + w.h;
     }
 };
 
-__device__ __forceinline__ void build_sched(Sched& s, const AtParams& p) {
+// One thread: the tiles of every sequence from the lengths and row offsets in s.S and s.row0.
+__device__ __forceinline__ void finish_sched(Sched& s, const AtParams& p) {
     s.B = p.B; s.H = p.H;
-    int u = 0;
-    s.row0[0] = p.row_off[0];
+    int u = 0, longest = 0;
     for (int b = 0; b < p.B; ++b) {
-        s.row0[b + 1] = p.row_off[b + 1];
         // a device-held length that breaks the caller's contract must not turn into a negative or unbounded tile
         // count: it is brought inside the cache (the tensor maps read zeros past the cache's end anyway)
-        const int rows_b = min(max(s.row0[b + 1] - s.row0[b], 0), AT_ROWS);
-        s.S[b] = min(max(p.seq_len[b], 0), max(p.max_seq - rows_b, 0));
-        const int total = s.S[b] + rows_b;
-        s.tiles[b] = (total + AT_KEYS - 1) / AT_KEYS;
+        const int rows_b = s.rows(b, p.rows_cap);
+        s.S[b] = min(max(s.S[b], 0), max(p.max_seq - rows_b, 0));
+        s.tiles[b] = (s.S[b] + rows_b + AT_KEYS - 1) / AT_KEYS;
+        longest = max(longest, s.tiles[b]);
         s.first[b] = u;
         u += s.tiles[b] * p.H;
     }
     s.first[p.B] = u;
+    s.head = -1; s.whole = 0;
+    if (p.cluster > 0) return;
+    // Whole heads need no merge; equal shares are shorter when a head is much longer than a share.  A merge (pieces to L2 and
+    // back in the second kernel) takes about as long as six tiles.
+    s.whole = p.B * p.H <= p.streams && longest <= u / p.streams + 6;
 }
-// The calling CTA's units.  Without clusters: equal contiguous ranges of all units.  With clusters (one sequence,
-// one head per cluster): the head's tiles are shared out among the CTAs of the cluster.
-__device__ __forceinline__ void build_range(Sched& s, const AtParams& p) {
-    if (p.cluster > 1) {
-        const int head = blockIdx.x / p.cluster, rank = blockIdx.x % p.cluster, T = s.tiles[0];
-        // shares rounded so that the extra tiles go to the FIRST CTAs: their tiles are cached rows that are already
-        // on their way when the previous kernel ends, while the last CTA has the tile with this step's rows, the
-        // masks and the padding to deal with
-        s.u_begin = head * T + (T * rank + p.cluster - 1) / p.cluster;
-        s.u_end = head * T + (T * (rank + 1) + p.cluster - 1) / p.cluster;
+// A batch's schedule, by all threads of the CTA; complete after the caller's next __syncthreads.
+__device__ __forceinline__ void build_batch_sched(Sched& s, const AtParams& p) {
+    for (int b = threadIdx.x; b <= p.B; b += blockDim.x) s.row0[b] = p.row_off[b];
+    for (int b = threadIdx.x; b < p.B; b += blockDim.x) s.S[b] = p.seq_len[b];
+    __syncthreads();
+    if (threadIdx.x == 0) finish_sched(s, p);
+}
+// The units of stream `st` of CTA `cta` (one thread per stream).  One sequence: the head's tiles are shared out among the
+// streams of its cluster, rounded so that the extra tiles go to the FIRST streams: their tiles are cached rows that are
+// already on their way when the previous kernel ends, while the last stream has the tile with this step's rows, the masks
+// and the padding to deal with.  A batch: equal contiguous ranges of all units, or whole heads, long next to short ones when
+// the lengths grow along the batch (the pieces of a prompt): stream 0 of CTA c takes head c, stream 1 the c-th from the end.
+__device__ __forceinline__ void build_range(Sched& s, const AtParams& p, int cta, int st) {
+    int begin = 0, end = 0;
+    if (p.cluster > 0) {
+        const int shift = __ffs(AT_STREAMS * p.cluster) - 1, n = 1 << shift;      // streams of a cluster: 2, 4 or 8
+        const int i = (AT_STREAMS * cta + st) & (n - 1), head = (AT_STREAMS * cta) >> shift, T = s.tiles[0];
+        begin = head * T + ((T * i + n - 1) >> shift);
+        end = head * T + ((T * (i + 1) + n - 1) >> shift);
+        s.head = head;
+    } else if (s.whole) {
+        const int heads = p.B * p.H, ctas = p.streams / AT_STREAMS, seg = st == 0 ? cta : heads - 1 - cta;
+        if (st == 0 ? cta < heads : seg >= ctas) {
+            const int b = seg / p.H, h = seg % p.H;
+            begin = s.first[b] + h * s.tiles[b];
+            end = begin + s.tiles[b];
+        }
     } else {
-        const long long U = s.first[p.B];
-        s.u_begin = (int)(U * blockIdx.x / gridDim.x);
-        s.u_end = (int)(U * (blockIdx.x + 1) / gridDim.x);
+        const unsigned U = s.first[p.B], n = p.streams, i = AT_STREAMS * cta + st;
+        if (U < (1u << 22)) {                                // n < 2^9: the products fit 32 bits, whose division is several times cheaper
+            begin = (int)(U * i / n);
+            end = (int)(U * (i + 1) / n);
+        } else {
+            begin = (int)((unsigned long long)U * i / n);
+            end = (int)((unsigned long long)U * (i + 1) / n);
+        }
     }
+    s.u_begin[st] = begin; s.u_end[st] = end;
 }
 
-// PRECISE: the probabilities go to the second product as a bf16 pair hi + lo (lo = the rounding error of hi, kept in
-// the tile's own score buffer once the scores are in registers), so the product sees ~16 mantissa bits of P.  A
-// single bf16 P costs ~1e-3 of relative error in the output whatever the number of keys (the output of near-uniform
-// attention is a mean of n values and the rounding errors of its n weights do not average out any faster than it
-// does); inside a deep decoder that error flips the bf16 roundings of the next layers' K/V rows and grows with depth.
-template <int AT_SPLIT, bool PRECISE>
-__global__ void __launch_bounds__(at_threads(AT_SPLIT), 1) tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q,
+// PRECISE: the probabilities go to the second product as a bf16 pair hi + lo (lo = the rounding error of hi, stored behind
+// hi), so the product sees ~16 mantissa bits of P.  A single bf16 P costs ~1e-3 of relative error in the output whatever the
+// number of keys (the output of near-uniform attention is a mean of n values and the rounding errors of its n weights do
+// not average out any faster than it does); inside a deep decoder that error flips the bf16 roundings of the next layers'
+// K/V rows and grows with depth.
+template <bool WIDE, bool PRECISE>
+__global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                           const __grid_constant__ CUtensorMap map_k,
                                                                           const __grid_constant__ CUtensorMap map_v,
                                                                           const AtParams p) {
-    constexpr int AT_KPT = 128 / AT_SPLIT;        // keys of a tile, and head_dim columns of O, per thread
-    constexpr int AT_SM_WARPS = 4 * AT_SPLIT;     // warp w owns TMEM lanes 32*(w%4).. and column group w/4
-    constexpr int AT_SM_THREADS = 32 * AT_SM_WARPS;
-    constexpr int AT_W_COPY = AT_SM_WARPS, AT_W_MMA = AT_SM_WARPS + 1;
-    constexpr int AT_THREADS = at_threads(AT_SPLIT);
-    static_assert(AT_KPT == 32 || AT_KPT == 64, "column groups are read with 32- or 64-column tensor-memory loads");
+    constexpr int ROWS = WIDE ? 128 : 64;                    // rows of a stream
+    constexpr int ROW_GROUPS = ROWS / 32, PARTS = AT_STREAM_WARPS / ROW_GROUPS;      // warps of 32 rows; threads that share a row
+    constexpr int GROUPS = 4 / PARTS;                        // 32-key groups of a tile, and 32-column groups of O, per thread
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[B_COUNT];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     __shared__ Sched sched;
-    __shared__ float pair_max[2][AT_SPLIT][AT_ROWS], pair_sum[2][AT_SPLIT][AT_ROWS];      // [parity][column group][row]
-    __shared__ float piece_m[AT_ROWS], piece_l[AT_ROWS];                     // this CTA's piece of a head shared by a cluster
+    __shared__ float part_max[2][AT_STREAMS][PARTS][ROWS], part_sum[AT_STREAMS][PARTS][ROWS];      // [parity][stream][column group][row]
+    __shared__ float piece_m[AT_STREAMS][ROWS], piece_l[AT_STREAMS][ROWS];      // this CTA's pieces of a head shared by a cluster
+    __shared__ __align__(16) float2 sum_ml[ROWS], peer_ml[4][ROWS];             // (max, sum) of their sum; of every CTA's
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    const uint32_t q_smem = base, ring_smem = base + AT_TILE;
+    // K slot of a stream; its V slot lies behind it
+    auto kv_smem = [&](int st) { return base + (uint32_t)(at_q_tiles(WIDE) + 2 * st) * AT_TILE; };
     const uint32_t bar0 = smem_u32(&bars[0]);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    pdl_launch_dependents();
+    if (p.in_chain) pdl_launch_dependents();
     TRJ_TL_DECL;
     if (threadIdx.x == 32) {                                 // have the tensor maps on their way before the first copy needs them
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+        prefetch_tensormap(&map_q);
+        prefetch_tensormap(&map_k);
+        prefetch_tensormap(&map_v);
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 64) {
         abort_flag = 0;
         for (int i = 0; i < B_COUNT; ++i)
-            mbar_init(bar(i), (i == B_P_READY || i == B_P_READY + 1 || i == B_O_FREE) ? AT_SM_THREADS : 1);
+            mbar_init(bar(i), (i >= B_P_READY && i < B_P_READY + AT_STREAMS) || (i >= B_O_FREE && i < B_O_FREE + AT_STREAMS) ? AT_STREAM_WARPS
+                              : i == B_PEERS && p.cluster > 0 ? p.cluster : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == AT_W_MMA) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    if (warp == AT_W_MMA) tmem_alloc(smem_u32(&tmem_base_slot), 512u);
+    for (int i = threadIdx.x; i < AT_STREAMS * ROWS; i += AT_THREADS) piece_m[i / ROWS][i % ROWS] = -INFINITY;       // no piece yet
     // Barriers, TMEM and the schedule are set up while the previous kernel may still run: the batch geometry is
     // older than the chain this kernel is launched in.  So are the cache rows below seq_len, which the copy thread
-    // starts to fetch before it waits; everything else (q, the tree's own K/V rows) is touched after the wait.
-    if (threadIdx.x == 0) { build_sched(sched, p); build_range(sched, p); }
-    if (threadIdx.x < AT_ROWS) piece_m[threadIdx.x] = -INFINITY;             // no piece yet
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    // starts to fetch before it waits; everything else (q, the tree's own K/V rows) is touched after the wait.  Outside a chain
+    // nothing is known of the previous kernel: all of this waits for it, and the merge kernel is let go only then.
+    if (!p.in_chain) { pdl_wait(); pdl_launch_dependents(); }
+    if (p.cluster > 0) {                                     // one sequence: one thread, one trip to memory
+        if (threadIdx.x == 0) {
+            const int first = p.row_off[0], last = p.row_off[1], len = p.seq_len[0];
+            sched.row0[0] = first; sched.row0[1] = last; sched.S[0] = len;
+            finish_sched(sched, p);
+            for (int st = 0; st < AT_STREAMS; ++st) build_range(sched, p, blockIdx.x, st);
+        }
+    } else {
+        build_batch_sched(sched, p);
+        __syncthreads();
+        if (threadIdx.x < AT_STREAMS) build_range(sched, p, blockIdx.x, threadIdx.x);
+    }
+    tc_fence_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc_fence_after();
+    if (p.cluster > 1) cluster_arrive_relaxed();             // the barriers exist (fenced above); waited for before the merge
     // Every role works out its first segment before it waits for the previous kernel (one thread's integer
     // divisions and address arithmetic take a microsecond that would otherwise sit on the critical path).
     const uint32_t tmem = tmem_base_slot;
-    // TMEM columns: S buffers 0-127 and 128-255, O 256-383, P buffers (bf16 pairs, 64 columns each) 384-447 and 448-511
-    const uint32_t tmem_s[2] = {tmem, tmem + 128}, tmem_o = tmem + 256, tmem_p[2] = {tmem + 384, tmem + 448};
-    const int u_begin = sched.u_begin, u_end = sched.u_end;
-    // With clusters every CTA leaves its piece in its own shared memory, and after a cluster barrier each CTA
-    // merges a slice of head_dim from all pieces.
-    float* piece_o = reinterpret_cast<float*>(base_ptr + AT_TILE);          // [row][AT_PIECE_STRIDE], over the K/V ring once it is idle
+    // TMEM columns: scores (then P) of stream 0 0-127, of stream 1 128-255; O of stream 0 256-383, of stream 1 384-511
+    const uint32_t tmem_s0 = tmem, tmem_o0 = tmem + 256;
+    const int n0 = sched.u_end[0] - sched.u_begin[0], n1 = sched.u_end[1] - sched.u_begin[1];      // tiles of each stream
+    // Q of a stream: its own tile, or its half of the one tile (64 rows of 128 bytes into each sub-tile)
+    auto q_rows_smem = [&](int st) { return WIDE ? base + st * AT_TILE : base + (uint32_t)st * 64u * 128u; };
+    auto load_q = [&](int st, const Where& w) {
+        mbar_expect_tx(bar(B_Q_FULL + st), ROWS * AT_D * 2);
+        tma_load_2d(q_rows_smem(st), &map_q, w.h * AT_D, sched.row0[w.b], bar(B_Q_FULL + st));
+        tma_load_2d(q_rows_smem(st) + AT_SUB, &map_q, w.h * AT_D + 64, sched.row0[w.b], bar(B_Q_FULL + st));
+    };
 
-    if (warp == AT_W_COPY) {
+    if (warp >= AT_W_COPY && warp < AT_W_MMA) {
         if (elect_one()) {
-            // ------------------------------------------------ TMA producer
-            int g = 0, e = 0;
-            bool ok = true;
-            bool waited = false;                             // for the previous kernel (see above)
+            // ------------------------------------------------ TMA producer of a stream
+            const int st = warp - AT_W_COPY, n = st == 0 ? n0 : n1, u0 = sched.u_begin[st];
+            bool ok = true, waited = false;                  // for the previous kernel (see above)
             const uint64_t kv_policy = l2_evict_first_policy();
             if (!p.early_ok) { pdl_wait(); waited = true; }
-            for (int u = u_begin; u < u_end && ok;) {
-                Where w; sched.locate(u, w);
-                const int t_end = min(w.tiles, w.t + (u_end - u));
-                // Q of this segment (after the previous segment's S = Q.K^T products have finished)
-                auto load_q = [&]() -> bool {
-                    if (!mbar_wait(bar(B_Q_EMPTY), (uint32_t)(e & 1) ^ 1u, &abort_flag, p.status)) return false;
-                    mbar_expect_tx(bar(B_Q_FULL), AT_TILE);
-                    tma_load_2d(q_smem, &map_q, w.h * AT_D, sched.row0[w.b], bar(B_Q_FULL));
-                    tma_load_2d(q_smem + AT_SUB, &map_q, w.h * AT_D + 64, sched.row0[w.b], bar(B_Q_FULL));
-                    return true;
-                };
-                // the first segment's Q is requested by the MMA thread as soon as the previous kernel is done, so
-                // that it does not queue behind the cache tiles this thread asks for ahead of the wait
-                if (e > 0) { ok = load_q(); if (!ok) break; }
-                const int cache_row0 = ((p.shared_cache ? 0 : w.b) * p.Hkv + w.h / p.group) * p.max_seq;
-                const int old_tiles = w.S / AT_KEYS;          // tiles that hold cached rows only
-                for (int t = w.t; t < t_end && ok; ++t, ++g) {
-                    for (int kv = 0; kv < 2 && ok; ++kv) {
-                        // rows of this step, or a ring slot that is only freed once Q has arrived: bounded waits
-                        // must not start while the previous kernel may still run
-                        if (!waited && (t >= old_tiles || 2 * g + kv >= AT_RING)) { pdl_wait(); waited = true; }
-                        const int slot = (2 * g + kv) % AT_RING;
-                        const uint32_t phase = (uint32_t)((2 * g + kv) / AT_RING) & 1u;
-                        ok = mbar_wait(bar(B_KV_EMPTY + slot), phase ^ 1u, &abort_flag, p.status);
-                        if (!ok) break;
-                        const uint32_t dst = ring_smem + slot * AT_TILE;
-                        mbar_expect_tx(bar(B_KV_FULL + slot), AT_TILE);
-                        const CUtensorMap* map = kv ? &map_v : &map_k;
-                        tma_load_2d_hint(dst, map, 0, cache_row0 + t * AT_KEYS, bar(B_KV_FULL + slot), kv_policy);
-                        tma_load_2d_hint(dst + AT_SUB, map, 64, cache_row0 + t * AT_KEYS, bar(B_KV_FULL + slot), kv_policy);
-                    }
+            Where w = {};
+            int row0 = 0, seg = 0;                           // first cache row of the head; segments begun before this one
+            auto load = [&](const CUtensorMap* map, int full, int empty, uint32_t dst, int g) {
+                if (ok && g > 0) ok = mbar_wait(bar(empty + st), (uint32_t)(g - 1) & 1u, &abort_flag, p.status);
+                if (!ok) return;
+                mbar_expect_tx(bar(full + st), AT_TILE);
+                tma_load_2d_hint(dst, map, 0, row0 + w.t * AT_KEYS, bar(full + st), kv_policy);
+                tma_load_2d_hint(dst + AT_SUB, map, 64, row0 + w.t * AT_KEYS, bar(full + st), kv_policy);
+            };
+            for (int g = 0; g < n && ok; ++g) {
+                const bool enter = g == 0 || w.t + 1 == w.tiles;
+                if (enter) {
+                    sched.locate(u0 + g, w, ROWS);
+                    row0 = ((p.shared_cache ? 0 : w.b) * p.Hkv + (p.group == 1 ? w.h : w.h / p.group)) * p.max_seq;
+                } else {
+                    ++w.t;
                 }
-                if (!waited) { pdl_wait(); waited = true; }  // the next segment's Q comes from the previous kernel
-                u += t_end - w.t;
-                ++e;
+                // rows of this step, or a slot that is only freed once Q has arrived: bounded waits must not start while the
+                // previous kernel may still run
+                if (!waited && (g > 0 || (w.t + 1) * AT_KEYS > w.S)) { pdl_wait(); waited = true; }
+                if (enter && g > 0) {                        // a new segment: its Q once the S products of the last one have finished
+                    ok = mbar_wait(bar(B_Q_EMPTY + st), (uint32_t)(seg & 1), &abort_flag, p.status);
+                    if (!ok) break;
+                    ++seg;
+                    load_q(st, w);                           // (the first segment's Q is requested by the MMA thread)
+                }
+                load(&map_k, B_K_FULL, B_K_EMPTY, kv_smem(st), g);
+                load(&map_v, B_V_FULL, B_V_EMPTY, kv_smem(st) + AT_TILE, g);
             }
             if (!waited) pdl_wait();
         }
-    } else if (warp == AT_W_MMA) {
+    } else if (warp >= AT_W_MMA) {
         if (elect_one()) {
-            // ------------------------------------------------ MMA issuer
-            // S = Q.K^T: both K-major from shared memory, 128 x 128.  O += P.V: P from TMEM, V MN-major, 128 x 128.
-            const uint32_t idesc_qk = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(AT_KEYS >> 3) << 17) | ((uint32_t)(AT_ROWS >> 4) << 24);
-            const uint32_t idesc_pv = idesc_qk | (1u << 16);
-            int g = 0, e = 0;
-            bool ok = true;
-            auto issue_qk = [&](int gg) -> bool {
-                const int slot = (2 * gg) % AT_RING;
-                if (!mbar_wait(bar(B_KV_FULL + slot), (uint32_t)((2 * gg) / AT_RING) & 1u, &abort_flag, p.status)) return false;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t k_smem = ring_smem + slot * AT_TILE;
-                // 8 x 16 elements of head_dim: two sub-tiles of four steps
-                const uint64_t q_desc = desc_kmajor_sw128(q_smem), k_desc = desc_kmajor_sw128(k_smem);
-                umma8_qk(tmem_s[gg & 1], (uint32_t)q_desc, (uint32_t)k_desc, (uint32_t)(q_desc >> 32), idesc_qk);
-                umma_commit(bar(B_S_FULL + (gg & 1)));
-                umma_commit(bar(B_KV_EMPTY + slot));
-                return true;
+            // ------------------------------------------------ MMA issuer of a stream
+            // S = Q.K^T: both K-major from shared memory, 128 x 128.  O += P.V: P from TMEM, V MN-major, 128 x 128.  The products of
+            // one thread run in the order of their issue, so the scores of a tile may replace the P that the product
+            // before them reads.  K and V of a step are waited for before P is, so that between P and the next scores there
+            // is nothing but the products themselves.
+            const int st = warp - AT_W_MMA, n = st == 0 ? n0 : n1, u0 = sched.u_begin[st];
+            const uint32_t idesc_qk = idesc_bf16(AT_LANES, AT_KEYS), idesc_pv = idesc_qk | (1u << 16);
+            const uint32_t d = tmem_o0 + 128 * st, a = tmem_s0 + 128 * st;
+            // 64-row streams: all 128 rows of the shared Q tile
+            const uint64_t q_desc = desc_kmajor_sw128(WIDE ? base + st * AT_TILE : base);
+            bool ok = n > 0;
+            Where w = {};
+            int in_seg = 0, seg = 0;                         // tiles left of the segment, this one included; segments begun before it
+            if (ok) { sched.locate(u0, w, ROWS); in_seg = min(w.tiles - w.t, n); }
+            pdl_wait();
+            const uint64_t k_desc = desc_kmajor_sw128(kv_smem(st)), v_desc = desc_mnmajor(kv_smem(st) + AT_TILE);
+            auto issue_qk = [&](bool last) {                 // 8 x 16 elements of head_dim: two sub-tiles of four steps
+                umma8_qk(a, (uint32_t)q_desc, (uint32_t)k_desc, (uint32_t)(q_desc >> 32), idesc_qk);
+                umma_commit(bar(B_S_FULL + st));
+                umma_commit(bar(B_K_EMPTY + st));
+                if (last) umma_commit(bar(B_Q_EMPTY + st));
             };
-            for (int u = u_begin; u < u_end && ok;) {
-                Where w; sched.locate(u, w);
-                const int n_tiles = min(w.tiles - w.t, u_end - u);
-                const int g0 = g, g1 = g + n_tiles;
-                if (e == 0) {                                // first segment: Q as soon as the previous kernel is done
-                    pdl_wait();
-                    mbar_expect_tx(bar(B_Q_FULL), AT_TILE);
-                    tma_load_2d(q_smem, &map_q, w.h * AT_D, sched.row0[w.b], bar(B_Q_FULL));
-                    tma_load_2d(q_smem + AT_SUB, &map_q, w.h * AT_D + 64, sched.row0[w.b], bar(B_Q_FULL));
+            if (ok) {
+                // the first segment's Q: requested here, so that it does not queue behind the cache tiles that the copy thread
+                // asks for ahead of the wait
+                load_q(st, w);
+                ok = mbar_wait(bar(B_K_FULL + st), 0u, &abort_flag, p.status) && mbar_wait(bar(B_Q_FULL + st), 0u, &abort_flag, p.status);
+                if (ok) { tc_fence_after(); issue_qk(in_seg == 1); }
+            }
+            bool first = true;                               // the tile at hand is the first of its segment
+            for (int g = 0; g < n && ok; ++g) {
+                const bool last = --in_seg == 0, more = g + 1 < n, first_now = first;
+                first = last;
+                ok = mbar_wait(bar(B_V_FULL + st), (uint32_t)g & 1u, &abort_flag, p.status);
+                if (ok && first_now && seg > 0) ok = mbar_wait(bar(B_O_FREE + st), (uint32_t)(seg - 1) & 1u, &abort_flag, p.status);
+                if (ok && last && more) {
+                    sched.locate(u0 + g + 1, w, ROWS);
+                    in_seg = min(w.tiles - w.t, n - g - 1);
+                    ++seg;
+                    ok = mbar_wait(bar(B_Q_FULL + st), (uint32_t)seg & 1u, &abort_flag, p.status);
                 }
-                ok = mbar_wait(bar(B_Q_FULL), (uint32_t)(e & 1), &abort_flag, p.status);
+                if (ok && more) ok = mbar_wait(bar(B_K_FULL + st), (uint32_t)(g + 1) & 1u, &abort_flag, p.status);
+                if (ok) ok = mbar_wait(bar(B_P_READY + st), (uint32_t)g & 1u, &abort_flag, p.status);
                 if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                ok = issue_qk(g0);
-                for (g = g0; g < g1 && ok; ++g) {
-                    if (g + 1 < g1) ok = issue_qk(g + 1);
-                    else umma_commit(bar(B_Q_EMPTY));        // every S product of the segment has been issued
-                    if (!ok) break;
-                    ok = mbar_wait(bar(B_P_READY + (g & 1)), (uint32_t)(g >> 1) & 1u, &abort_flag, p.status);
-                    if (ok && g == g0 && e > 0) ok = mbar_wait(bar(B_O_FREE), (uint32_t)((e - 1) & 1), &abort_flag, p.status);
-                    const int slot = (2 * g + 1) % AT_RING;
-                    if (ok) ok = mbar_wait(bar(B_KV_FULL + slot), (uint32_t)((2 * g + 1) / AT_RING) & 1u, &abort_flag, p.status);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t v_smem = ring_smem + slot * AT_TILE;
-                    // 8 x 16 keys; P comes straight from TMEM
-                    const uint64_t v_desc = desc_mnmajor(v_smem);
-                    umma8_pv(tmem_o, tmem_p[g & 1], (uint32_t)v_desc, (uint32_t)(v_desc >> 32), idesc_pv, g > g0 ? 1u : 0u);
-                    if constexpr (PRECISE)                   // the low halves of P sit in the first 64 columns of the tile's S buffer
-                        umma8_pv(tmem_o, tmem_s[g & 1], (uint32_t)v_desc, (uint32_t)(v_desc >> 32), idesc_pv, 1u);
-                    umma_commit(bar(B_P_FREE + (g & 1)));
-                    umma_commit(bar(B_KV_EMPTY + slot));
-                }
-                if (ok) umma_commit(bar(B_O_READY));
-                u += n_tiles;
-                ++e;
+                tc_fence_after();
+                umma8_pv(d, a, (uint32_t)v_desc, (uint32_t)(v_desc >> 32), idesc_pv, first_now ? 0u : 1u);
+                if constexpr (PRECISE)                       // the low halves lie 16 columns behind
+                    umma8_pv(d, a + 16, (uint32_t)v_desc, (uint32_t)(v_desc >> 32), idesc_pv, 1u);
+                umma_commit(bar(B_V_EMPTY + st));
+                if (last) umma_commit(bar(B_O_READY + st));  // the last commit of a stream: the epilogue, and the CTA's exit, wait for it
+                if (more) issue_qk(in_seg == 1);
             }
         }
     } else {
         // ------------------------------------------------ softmax + epilogue
-        // Warp w owns rows 32*(w%4) .. +31 (its TMEM lanes) and key / head_dim columns AT_KPT*(w/4) .. +AT_KPT-1, so
-        // AT_SPLIT threads share a row and exchange their maxima and sums through shared memory.
-        const int rg = warp & 3, part = warp >> 2;
+        // A warp owns 32 rows of a stream (its TMEM lanes are 32 * (warp % 4) ..) and the 32-column groups GROUPS * part .. of the
+        // scores and of O; PARTS threads share a row and exchange their maxima and sums through shared memory.
+        const int lane_group = warp & 3;
+        const int st = WIDE ? (warp >> 2) & 1 : lane_group >> 1, part = WIDE ? warp >> 3 : warp >> 2;
+        const int rg = WIDE ? lane_group : lane_group & 1;
         const int row = rg * 32 + lane;
-        const uint32_t lane_addr = (uint32_t)(rg * 32) << 16;
-        const uint32_t col0 = (uint32_t)part * AT_KPT;
-        const uint32_t pair_bar = 1 + rg;                    // named barrier of the warps of a row group
+        const uint32_t lane_addr = (uint32_t)(lane_group * 32) << 16;
+        const uint32_t scores = tmem_s0 + 128 * st + lane_addr + 32 * GROUPS * part, accum = tmem_o0 + 128 * st + lane_addr + 32 * GROUPS * part;
+        const int col0 = 32 * GROUPS * part;                 // first key of a tile, first column of head_dim of this thread
+        const uint32_t pair_bar = 1 + st * ROW_GROUPS + rg;  // named barrier of the warps that share 32 rows
+        const int stream_thread = (part * ROW_GROUPS + rg) * 32 + lane;
+        const int u_end = sched.u_end[st];
+        // A warp whose wait gave up arrives where the others of its row group may already be waiting for it.
+        auto leave_row_group = [&](bool in_use, int barriers) {
+            for (int i = 0; in_use && i < barriers; ++i) asm volatile("bar.arrive %0, %1;" ::"r"(pair_bar), "n"(32 * PARTS) : "memory");
+        };
         int g = 0, e = 0;
         bool ok = true;
-        for (int u = u_begin; u < u_end && ok;) {
-            Where w; sched.locate(u, w);
+        for (int u = sched.u_begin[st]; u < u_end && ok;) {
+            Where w; sched.locate(u, w, ROWS);
             const int n_tiles = min(w.tiles - w.t, u_end - u);
             const int g0 = g, g1 = g + n_tiles;
             const bool live = row < w.rows;
-            const bool group_live = rg * 32 < w.rows;        // same for both warps of the pair
-            const int grow = sched.row0[w.b] + row;           // global row (valid when live)
+            const bool group_live = rg * 32 < w.rows;        // the same for all warps that share the rows
+            const int grow = sched.row0[w.b] + row;          // global row (valid when live)
             uint64_t m0 = 0, m1 = 0;
             if (live) {
                 m0 = p.anc[(size_t)grow * p.anc_words];
@@ -472,161 +467,128 @@ __global__ void __launch_bounds__(at_threads(AT_SPLIT), 1) tree_attention_tc_ker
             const int total = w.S + w.rows;
             float m_ref = -INFINITY, l_sum = 0.f;
             if (e == 0) { pdl_wait(); TRJ_TL_BEGIN(TRJ_TL_ATTENTION); }      // the ancestor masks above are older than the chain
-            for (g = g0; g < g1 && ok; ++g) {
+            for (g = g0; g < g1; ++g) {
                 const int key0 = (w.t + (g - g0)) * AT_KEYS;
                 const bool edge = key0 + AT_KEYS > w.S;      // the tile reaches tree rows or the end of the keys
-                float s[AT_KPT];
-                float mt = -INFINITY;
+                // scores complete, and with them every product issued before: the last tile's P has been read, O may be touched
+                ok = __all_sync(0xffffffffu, mbar_wait(bar(B_S_FULL + st), (uint32_t)(g & 1), &abort_flag, p.status));
+                if (!ok) { leave_row_group(group_live, 1); break; }
+                tc_fence_after();
                 if (group_live) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(bar(B_S_FULL + (g & 1)), (uint32_t)(g >> 1) & 1u, &abort_flag, p.status));
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if constexpr (AT_KPT == 64) tmem_ld64(tmem_s[g & 1] + lane_addr + col0, s);
-                    else tmem_ld32(tmem_s[g & 1] + lane_addr + col0, s);
+                    float s[32], mt = -INFINITY;
+                    // bit c of (vis0, vis1) = visibility of key key0 + c for this row: tree row tt = key0 + c - S
+                    // is visible if tt < 0 (prefix) or if bit tt of the row's ancestor mask is set
+                    uint64_t vis0 = m0, vis1 = m1;
                     if (edge) {
-                        // bit c of (vis0, vis1) = visibility of key key0 + c for this row: tree row tt = key0 + c - S
-                        // is visible if tt < 0 (prefix) or if bit tt of the row's ancestor mask is set
-                        uint64_t vis0 = m0, vis1 = m1;
                         const int d = key0 - w.S;            // -127 .. 127 on an edge tile
                         if (d >= 0) shr128(vis0, vis1, d); else shl128_fill(vis0, vis1, -d);
-                        const uint64_t vis = (col0 < 64 ? vis0 : vis1) >> (col0 & 63u);      // this thread's AT_KPT keys
-#pragma unroll
-                        for (int i = 0; i < AT_KPT; ++i) if (!((vis >> i) & 1ull)) s[i] = -INFINITY;
                     }
-                    {   // four independent chains instead of one 64-long dependency chain
-                        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                    auto load_scores = [&](int grp) {        // 32 scores of this row, masked
+                        tmem_ld32(scores + 32 * grp, s);
+                        if (edge) {
+                            const int c0 = col0 + 32 * grp;
+                            const uint32_t vis = (uint32_t)((c0 < 64 ? vis0 : vis1) >> (c0 & 63));
 #pragma unroll
-                        for (int i = 0; i < AT_KPT; i += 4) {
+                            for (int i = 0; i < 32; ++i) if (!((vis >> i) & 1u)) s[i] = -INFINITY;
+                        }
+                    };
+#pragma unroll
+                    for (int grp = 0; grp < GROUPS; ++grp) {
+                        load_scores(grp);                    // the last group stays in registers
+                        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // independent chains
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
                             mx[0] = fmaxf(mx[0], s[i]); mx[1] = fmaxf(mx[1], s[i + 1]);
                             mx[2] = fmaxf(mx[2], s[i + 2]); mx[3] = fmaxf(mx[3], s[i + 3]);
                         }
-                        mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                        mt = fmaxf(mt, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
                     }
-                    pair_max[g & 1][part][row] = mt;
-                    asm volatile("bar.sync %0, %1;" ::"r"(pair_bar), "n"(32 * AT_SPLIT) : "memory");
+                    part_max[g & 1][st][part][row] = mt;
+                    asm volatile("bar.sync %0, %1;" ::"r"(pair_bar), "n"(32 * PARTS) : "memory");
 #pragma unroll
-                    for (int q = 0; q < AT_SPLIT; ++q) mt = fmaxf(mt, pair_max[g & 1][q][row]);
+                    for (int q = 0; q < PARTS; ++q) mt = fmaxf(mt, part_max[g & 1][st][q][row]);
                     mt *= p.scale_log2;
-                }
-                // this tile's P buffer was last read by the P.V product of two tiles ago
-                if (g > 1) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_P_FREE + (g & 1)), ((uint32_t)(g >> 1) & 1u) ^ 1u, &abort_flag, p.status));
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (group_live) {
                     float factor = 1.f;
                     if (live && mt > -INFINITY) {
                         if (m_ref == -INFINITY) m_ref = mt;
                         else if (mt > m_ref + AT_RESCALE_GAP) { factor = fast_exp2(m_ref - mt); m_ref = mt; }
                     }
                     if (g > g0 && __any_sync(0xffffffffu, factor != 1.f)) {
-                        // O may only be touched once the previous P.V product has finished
-                        ok = __all_sync(0xffffffffu, mbar_wait(bar(B_P_FREE + ((g - 1) & 1)), (uint32_t)((g - 1) >> 1) & 1u, &abort_flag, p.status));
-                        if (!ok) break;
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         l_sum *= factor;
 #pragma unroll 1
-                        for (int c0 = 0; c0 < AT_KPT; c0 += 32) {
-                            float o[32];
-                            tmem_ld32(tmem_o + lane_addr + col0 + c0, o);
+                        for (int c0 = 0; c0 < 32 * GROUPS; c0 += 16) {
+                            uint32_t o[16];
+                            tmem_ld8(accum + c0, reinterpret_cast<float*>(o));
+                            tmem_ld8(accum + c0 + 8, reinterpret_cast<float*>(o) + 8);
+                            tmem_wait_ld();
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] *= factor;
-                            tmem_st32(tmem_o + lane_addr + col0 + c0, o);
+                            for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * factor);
+                            tmem_st16u(accum + c0, o);
+                            tmem_wait_st();
                         }
                     }
-                    // P = 2^(s * c - m_ref) as bf16 pairs into this tile's P buffer in TMEM (lane = row, one column
-                    // per two keys); masked scores are -inf and give exactly 0.  Rows past the tree store zeros.
+                    // P = 2^(s * c - m_ref) as bf16 over the scores it comes from (lane = row, one column per two keys, the low
+                    // halves 16 columns behind); masked scores are -inf and give exactly 0.  Lanes without a row keep their
+                    // scores: what they add up to is not looked at.
                     const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
-                    uint32_t packed[AT_KPT / 2];
-                    if (live) {
+#pragma unroll
+                    for (int k = GROUPS - 1; k >= 0; --k) {
+                        if (k < GROUPS - 1) load_scores(k);
+                        uint32_t hi[16], lo[16];
                         float ls[4] = {0.f, 0.f, 0.f, 0.f};  // independent partial sums
 #pragma unroll
-                        for (int i = 0; i < AT_KPT; i += 4) {
+                        for (int i = 0; i < 32; i += 2) {
                             const float a = fast_exp2(fmaf(s[i], p.scale_log2, -m_use));
                             const float b = fast_exp2(fmaf(s[i + 1], p.scale_log2, -m_use));
-                            const float c = fast_exp2(fmaf(s[i + 2], p.scale_log2, -m_use));
-                            const float d = fast_exp2(fmaf(s[i + 3], p.scale_log2, -m_use));
-                            ls[0] += a; ls[1] += b; ls[2] += c; ls[3] += d;
-                            packed[i >> 1] = pack_bf16(a, b);
-                            packed[(i >> 1) + 1] = pack_bf16(c, d);
+                            ls[i & 2] += a; ls[(i & 2) + 1] += b;
+                            hi[i >> 1] = pack_bf16(a, b);
+                            if constexpr (PRECISE)           // what the rounding to bf16 left: the halves of a pack are the floats' upper words
+                                lo[i >> 1] = pack_bf16(a - __uint_as_float(hi[i >> 1] << 16), b - __uint_as_float(hi[i >> 1] & 0xffff0000u));
                         }
                         l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < AT_KPT / 2; ++i) packed[i] = 0u;
+                        tmem_st16u(scores + 32 * k, hi);
+                        if constexpr (PRECISE) tmem_st16u(scores + 32 * k + 16, lo);
                     }
-                    if constexpr (AT_KPT == 64) tmem_st32u(tmem_p[g & 1] + lane_addr + (AT_KPT / 2) * part, packed);
-                    else tmem_st16u(tmem_p[g & 1] + lane_addr + (AT_KPT / 2) * part, packed);
-                    if constexpr (PRECISE) {
-                        // lo = p - bf16(p), recomputed from the scores 32 keys at a time (keeps the register count
-                        // down); every thread of the row group has its scores in registers since the exchange of
-                        // the maxima, so the S buffer may be overwritten
-#pragma unroll
-                        for (int c0 = 0; c0 < AT_KPT; c0 += 32) {
-                            uint32_t lo[16];
-                            if (live) {
-#pragma unroll
-                                for (int i = 0; i < 32; i += 2) {
-                                    const float a = fast_exp2(fmaf(s[c0 + i], p.scale_log2, -m_use));
-                                    const float b = fast_exp2(fmaf(s[c0 + i + 1], p.scale_log2, -m_use));
-                                    lo[i >> 1] = pack_bf16(a - bf16_round(a), b - bf16_round(b));
-                                }
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) lo[i] = 0u;
-                            }
-                            tmem_st16u(tmem_s[g & 1] + lane_addr + (AT_KPT / 2) * part + (c0 >> 1), lo);
-                        }
-                    }
+                    tmem_wait_st();
                 }
                 // keys past the end of the sequence hold whatever the cache holds: clear those V rows so
                 // that 0 * garbage cannot poison the product
                 if (key0 + AT_KEYS > total) {
-                    const int slot = (2 * g + 1) % AT_RING;
-                    ok = __all_sync(0xffffffffu, mbar_wait(bar(B_KV_FULL + slot), (uint32_t)((2 * g + 1) / AT_RING) & 1u, &abort_flag, p.status));
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar(B_V_FULL + st), (uint32_t)g & 1u, &abort_flag, p.status));
                     if (!ok) break;
-                    uint8_t* v_ptr = base_ptr + AT_TILE + slot * AT_TILE;
+                    uint8_t* v_ptr = base_ptr + (kv_smem(st) + AT_TILE - base);
                     const int first_bad = max(total - key0, 0);
-                    for (int i = first_bad * 8 + (int)threadIdx.x; i < AT_KEYS * 8; i += AT_SM_THREADS) {      // 16-byte chunks, both sub-tiles
+                    for (int i = first_bad * 8 + stream_thread; i < AT_KEYS * 8; i += 32 * AT_STREAM_WARPS) {      // 16-byte chunks, both sub-tiles
                         *reinterpret_cast<uint4*>(v_ptr + i * 16) = make_uint4(0, 0, 0, 0);
                         *reinterpret_cast<uint4*>(v_ptr + AT_SUB + i * 16) = make_uint4(0, 0, 0, 0);
                     }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the MMA reads V through the async proxy
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive(bar(B_P_READY + (g & 1)));
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_P_READY + st));
             }
             if (!ok) break;
             // ---- epilogue of the segment
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(B_O_READY), (uint32_t)(e & 1), &abort_flag, p.status));
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            ok = __all_sync(0xffffffffu, mbar_wait(bar(B_O_READY + st), (uint32_t)(e & 1), &abort_flag, p.status));
+            if (!ok) { leave_row_group(group_live, 2); break; }
+            tc_fence_after();
             if (group_live) {
-                pair_sum[e & 1][part][row] = l_sum;
-                asm volatile("bar.sync %0, %1;" ::"r"(pair_bar), "n"(32 * AT_SPLIT) : "memory");
+                part_sum[st][part][row] = l_sum;
+                asm volatile("bar.sync %0, %1;" ::"r"(pair_bar), "n"(32 * PARTS) : "memory");
                 float l_row = 0.f;
 #pragma unroll
-                for (int q = 0; q < AT_SPLIT; ++q) l_row += pair_sum[e & 1][q][row];     // the same order in every thread
-                const bool whole_seg = (w.t == 0 && n_tiles == w.tiles);
-                if (p.cluster > 1) {
-                    // all products that read the ring have finished (B_O_READY), and this CTA loads nothing more
-#pragma unroll 1
-                    for (int c0 = 0; c0 < AT_KPT; c0 += 32) {
-                        float o[32];
-                        tmem_ld32(tmem_o + lane_addr + col0 + c0, o);
-                        if (live) {
-                            float4* dst = reinterpret_cast<float4*>(piece_o + (size_t)row * AT_PIECE_STRIDE + col0 + c0);
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) dst[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-                        }
-                    }
-                    if (live && part == 0) { piece_m[row] = m_ref; piece_l[row] = l_row; }
-                } else if (whole_seg) {
+                for (int q = 0; q < PARTS; ++q) l_row += part_sum[st][q][row];       // the same order in every thread
+                if (p.cluster > 0) {
+                    // a piece of the head: O stays in TMEM until both streams are done (it goes where the ring is)
+                    if (live && part == 0) { piece_m[st][row] = m_ref; piece_l[st][row] = l_row; }
+                } else if (w.t == 0 && n_tiles == w.tiles) {
                     const float inv = live ? 1.f / l_row : 0.f;
                     const size_t off = ((size_t)grow * p.H + w.h) * AT_D + col0;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < AT_KPT; c0 += 32) {
+                    for (int c0 = 0; c0 < 32 * GROUPS; c0 += 32) {
                         float o[32];
-                        tmem_ld32(tmem_o + lane_addr + col0 + c0, o);
+                        tmem_ld32(accum + c0, o);
                         if (live) {
 #pragma unroll
                             for (int i = 0; i < 32; ++i) o[i] *= inv;
@@ -636,122 +598,201 @@ __global__ void __launch_bounds__(at_threads(AT_SPLIT), 1) tree_attention_tc_ker
                         }
                     }
                 } else {
-                    float* slot = p.slots + (size_t)(w.bh + (int)blockIdx.x) * AT_SLOT_FLOATS;
+                    float* slot = p.slots + (size_t)(w.bh + AT_STREAMS * (int)blockIdx.x + st) * AT_SLOT_FLOATS;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < AT_KPT; c0 += 32) {
+                    for (int c0 = 0; c0 < 32 * GROUPS; c0 += 32) {
                         float o[32];
-                        tmem_ld32(tmem_o + lane_addr + col0 + c0, o);
+                        tmem_ld32(accum + c0, o);
                         if (live) {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) slot[(size_t)(col0 + c0 + i) * AT_ROWS + row] = o[i];
+                            for (int i = 0; i < 32; ++i) slot[(size_t)(col0 + c0 + i) * AT_LANES + row] = o[i];
                         }
                     }
-                    if (live && part == 0) { slot[AT_D * AT_ROWS + row] = m_ref; slot[AT_D * AT_ROWS + AT_ROWS + row] = l_row; }
+                    if (live && part == 0) { slot[AT_D * AT_LANES + row] = m_ref; slot[AT_D * AT_LANES + AT_LANES + row] = l_row; }
                 }
+                // the sums are read before any warp of the row group writes the next segment's
+                asm volatile("bar.sync %0, %1;" ::"r"(pair_bar), "n"(32 * PARTS) : "memory");
             }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(bar(B_O_FREE));
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_O_FREE + st));
             u += n_tiles;
             ++e;
         }
     }
     __syncwarp();
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
     if (abort_flag) {                                        // let copies still in flight land before the CTA leaves
         for (int i = 0; i < 64; ++i) __nanosleep(1000);
         __syncthreads();
     }
-    if (p.cluster > 1) {
-        // Every CTA of the cluster gets here, with or without a piece, and also after a wait that gave up.
+    if (p.cluster > 0) {
+        // Merge of the head's pieces.  Every CTA of the cluster gets here, with or without pieces, and also after a wait that
+        // gave up.  First the CTA adds up its own two pieces; then each CTA gets a quarter (half) of head_dim of every
+        // other CTA's sum, by bulk copies into its shared memory, and finishes it.  (Reading all pieces of the
+        // cluster with ordinary loads took 6500 cycles for 64 rows and 13000 for 128; the copies and the final sum take 2300 and
+        // 4500.)
+        // Layout of a piece: four slices of 32 columns, [slice][row][8 x 16 bytes], the 16-byte chunks of a row permuted by
+        // row % 8 (no bank conflicts although rows are 128 bytes apart).
+        const int C = p.cluster, rank = blockIdx.x % C, head = blockIdx.x / C, slices = 4 / C;
+        const int rows = sched.rows(0, ROWS);
+        constexpr uint32_t SLICE = ROWS * 128, PIECE = 4 * SLICE;
+        const uint32_t peer_smem = base + PIECE;             // [CTA][its share of the slices]; behind the CTA's own sum
+        auto at = [&](uint32_t region, int slice, int row, int chunk) {      // everything lies over Q, K and V, which are idle
+            return reinterpret_cast<float4*>(base_ptr + (region - base) + slice * SLICE + row * 128 + ((chunk ^ (row & 7)) << 4));
+        };
         pdl_wait();                                          // threads that had no role have not waited yet
-        cluster_sync_all();                                  // all pieces are in place and visible
-        const int C = p.cluster, rank = blockIdx.x % C, head = blockIdx.x / C;
-        const int rows = sched.row0[1] - sched.row0[0], width = AT_D / C, groups = width / 4;
-        const uint32_t m_local = smem_u32(piece_m), l_local = smem_u32(piece_l), o_local = smem_u32(piece_o);
-        if (!abort_flag) {
-            for (int i = threadIdx.x; i < rows * groups; i += AT_THREADS) {
-                const int row = i / groups, col = rank * width + 4 * (i % groups);
-                // every piece's statistics and values are requested before any is used
-                float m_c[8], l_c[8], m_all = -INFINITY;
-                float4 o_c[8];
+        if (C > 1) {
+            cluster_wait();                                  // every CTA's barriers have been initialised
+            if (threadIdx.x < C) mbar_arrive_cluster(cluster_addr(bar(B_PEERS), threadIdx.x));      // this CTA's K and V are idle
+            if (threadIdx.x == 32) mbar_expect_tx(bar(B_RECEIVED), (uint32_t)(C - 1) * (slices * rows * 128 + ROWS * (uint32_t)sizeof(float2)));
+        }
+        // The own sum: stream 0's warps finish slices 0 and 1, stream 1's warps 2 and 3, each from its accumulator and what the
+        // other stream's warps left in shared memory.  The same lanes and columns as above.
+        const int lane_group = warp & 3, st = WIDE ? (warp >> 2) & 1 : lane_group >> 1, part = WIDE ? warp >> 3 : warp >> 2;
+        const int rg = WIDE ? lane_group : lane_group & 1, row = rg * 32 + lane;
+        const bool role = warp < AT_SM_WARPS && rg * 32 < rows, finishes = ((GROUPS * part) >> 1) == st, has_piece = (st == 0 ? n0 : n1) > 0;
+        const uint32_t accum = tmem_o0 + 128 * st + ((uint32_t)(lane_group * 32) << 16);
+        if (role && !finishes && has_piece) {
+#pragma unroll 1
+            for (int slice = GROUPS * part; slice < GROUPS * (part + 1); ++slice) {
+                float o[32];
+                tmem_ld32(accum + 32 * slice, o);
+                if (row < rows) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    if (c < C) {
-                        m_c[c] = ld_cluster(cluster_addr(m_local + 4u * row, c));
-                        l_c[c] = ld_cluster(cluster_addr(l_local + 4u * row, c));
-                        o_c[c] = ld_cluster4(cluster_addr(o_local + 4u * (uint32_t)(row * AT_PIECE_STRIDE + col), c));
-                    }
+                    for (int i = 0; i < 8; ++i) *at(base, slice, row, i) = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                 }
-#pragma unroll
-                for (int c = 0; c < 8; ++c) if (c < C) m_all = fmaxf(m_all, m_c[c]);
-                float l_all = 0.f;
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {                // pieces in ascending tile order; one without keys holds no data
-                    if (c >= C || m_c[c] == -INFINITY) continue;
-                    const float wgt = exp2f(m_c[c] - m_all);
-                    l_all = fmaf(l_c[c], wgt, l_all);
-                    acc.x = fmaf(o_c[c].x, wgt, acc.x); acc.y = fmaf(o_c[c].y, wgt, acc.y);
-                    acc.z = fmaf(o_c[c].z, wgt, acc.z); acc.w = fmaf(o_c[c].w, wgt, acc.w);
-                }
-                const float inv = 1.f / l_all;
-                const size_t off = ((size_t)(sched.row0[0] + row) * p.H + head) * AT_D + col;
-                store4_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
             }
         }
-        cluster_sync_all();                                  // nobody leaves while its piece may still be read
+        __syncthreads();
+        if (role && finishes) {
+            float w_own = 0.f, w_other = 0.f;                // a piece without keys (maximum -inf) holds no data
+            if (row < rows) {
+                const float m_own = piece_m[st][row], m_other = piece_m[st ^ 1][row], m = fmaxf(m_own, m_other);
+                if (m_own > -INFINITY) w_own = exp2f(m_own - m);
+                if (m_other > -INFINITY) w_other = exp2f(m_other - m);
+                if (part == 0)
+                    sum_ml[row] = make_float2(m, (w_own > 0.f ? piece_l[st][row] * w_own : 0.f) + (w_other > 0.f ? piece_l[st ^ 1][row] * w_other : 0.f));
+            }
+#pragma unroll 1
+            for (int slice = GROUPS * part; slice < GROUPS * (part + 1); ++slice) {
+                float o[32];
+                if (has_piece) tmem_ld32(accum + 32 * slice, o);
+                if (row < rows) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (w_own > 0.f) v = make_float4(o[4 * i] * w_own, o[4 * i + 1] * w_own, o[4 * i + 2] * w_own, o[4 * i + 3] * w_own);
+                        if (w_other > 0.f) {
+                            const float4 a = *at(base, slice, row, i);
+                            v.x = fmaf(a.x, w_other, v.x); v.y = fmaf(a.y, w_other, v.y); v.z = fmaf(a.z, w_other, v.z); v.w = fmaf(a.w, w_other, v.w);
+                        }
+                        *at(base, slice, row, i) = v;
+                    }
+                }
+            }
+        }
+        if (C > 1) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the bulk copies read what was just written
+            __syncthreads();
+            if (warp == 0 && mbar_wait_cluster(bar(B_PEERS), 0u, &abort_flag, p.status)) {
+                const int peer = lane / slices, slice = lane % slices;
+                if (peer < C && peer != rank) {
+                    if (rows > 0)
+                        bulk_copy_to_cluster(cluster_addr(peer_smem + (rank * slices + slice) * SLICE, peer), base + (peer * slices + slice) * SLICE,
+                                             rows * 128, cluster_addr(bar(B_RECEIVED), peer));
+                    if (slice == 0)
+                        bulk_copy_to_cluster(cluster_addr(smem_u32(&peer_ml[rank][0]), peer), smem_u32(&sum_ml[0]), ROWS * (uint32_t)sizeof(float2),
+                                             cluster_addr(bar(B_RECEIVED), peer));
+                }
+            }
+            mbar_wait_cluster(bar(B_RECEIVED), 0u, &abort_flag, p.status);
+            __syncwarp();
+            cluster_arrive_relaxed();                        // this CTA has what it needs of the others: no data to order
+        } else {
+            __syncthreads();
+        }
+        for (int i = threadIdx.x; i < rows * slices * 8; i += AT_THREADS) {
+            const int chunk = i & 7, slice = (i >> 3) & (slices - 1), row = (i >> 3) >> (__ffs(slices) - 1);
+            float2 ml[4];
+            float4 o[4];
+            float m_all = -INFINITY, l_all = 0.f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {                    // ascending CTAs, hence ascending tiles
+                if (c >= C) continue;
+                ml[c] = c == rank ? sum_ml[row] : peer_ml[c][row];
+                o[c] = *at(c == rank ? base : peer_smem, c * slices + slice, row, chunk);
+                m_all = fmaxf(m_all, ml[c].x);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (c >= C || ml[c].x == -INFINITY) continue;
+                const float wgt = exp2f(ml[c].x - m_all);
+                l_all = fmaf(ml[c].y, wgt, l_all);
+                acc.x = fmaf(o[c].x, wgt, acc.x); acc.y = fmaf(o[c].y, wgt, acc.y);
+                acc.z = fmaf(o[c].z, wgt, acc.z); acc.w = fmaf(o[c].w, wgt, acc.w);
+            }
+            const float inv = 1.f / l_all;
+            const size_t off = ((size_t)(sched.row0[0] + row) * p.H + head) * AT_D + (rank * slices + slice) * 32 + 4 * chunk;
+            store4_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+        }
+        if (C > 1) cluster_wait();                           // nobody leaves while its sum may still be copied
+        __syncthreads();
     }
-    if (warp == AT_W_MMA)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    if (warp == AT_W_MMA) tmem_dealloc(tmem, 512u);
 #ifdef TRJ_TIMELINE
-    if (threadIdx.x == 0 && u_begin >= u_end) tl_slot__ = ::trj::tl::begin(TRJ_TL_ATTENTION);   // a CTA without work never stamped its release
+    if (threadIdx.x == 0 && sched.u_begin[0] >= sched.u_end[0]) tl_slot__ = ::trj::tl::begin(TRJ_TL_ATTENTION);   // no work for this thread: it never stamped its release
 #endif
     TRJ_TL_END(TRJ_TL_ATTENTION);
 }
 
-// Merges the pieces of every (sequence, head) that more than one CTA worked on.  One CTA per
-// (sequence, head, 16-wide slice of head_dim), thread = row; pieces are taken in ascending CTA order.
+// Merges the pieces of every (sequence, head) that more than one stream worked on.  One CTA per
+// (sequence, head, 16-wide slice of head_dim), thread = row; pieces are taken in ascending stream order.
 constexpr int CB_COLS = 16;
-__global__ void __launch_bounds__(128) tree_attention_combine_kernel(const AtParams p, int grid_main) {
+__global__ void __launch_bounds__(128) tree_attention_combine_kernel(const AtParams p) {
     __shared__ Sched sched;
-    __shared__ float stage[AT_ROWS][CB_COLS + 1];
+    __shared__ float stage[AT_LANES][CB_COLS + 1];
     // the geometry (sequence lengths, row offsets) is not produced by the main kernel: work it out while that
     // kernel may still be running, and wait for its pieces only afterwards
     pdl_launch_dependents();
-    if (threadIdx.x == 0) build_sched(sched, p);
+    build_batch_sched(sched, p);
     __syncthreads();
+    if (sched.whole) { pdl_wait(); return; }                 // nothing was split
     const int bh = blockIdx.x, b = bh / p.H, h = bh % p.H, c0 = blockIdx.y * CB_COLS;
     const long long U = sched.first[p.B];
     const long long u0 = sched.first[b] + (long long)h * sched.tiles[b], u1 = u0 + sched.tiles[b];
-    // CTA c of the main kernel owns units [U*c/G, U*(c+1)/G): the owner of unit u is the largest c with U*c/G <= u
-    auto owner = [&](long long u) { return (int)(((u + 1) * grid_main + U - 1) / U - 1); };
+    if (u0 == u1) { pdl_wait(); return; }                    // a sequence without rows and keys
+    // stream c of the main kernel owns units [U*c/G, U*(c+1)/G): the owner of unit u is the largest c with U*c/G <= u
+    auto owner = [&](long long u) { return (int)(((u + 1) * p.streams + U - 1) / U - 1); };
     const int c_first = owner(u0), c_last = owner(u1 - 1);
-    const int row = threadIdx.x, rows = p.row_off[b + 1] - p.row_off[b];
+    const int row = threadIdx.x, rows = sched.rows(b, p.rows_cap);
     const bool live = row < rows;
-    // a CTA in between may own no unit at all (grid larger than the unit count): it wrote nothing
+    // a stream in between may own no unit at all (more streams than units): it wrote nothing
     auto has_piece = [&](int c) {
-        const long long rb = U * c / grid_main, re = U * (c + 1) / grid_main;
+        const long long rb = U * c / p.streams, re = U * (c + 1) / p.streams;
         return (rb > u0 ? rb : u0) < (re < u1 ? re : u1);
     };
     pdl_wait();
-    if (c_first == c_last) return;                           // written directly by its only CTA
+    if (c_first == c_last) return;                           // written directly by its only stream
     if (live) {
         float m_all = -INFINITY;
         for (int c = c_first; c <= c_last; ++c)
-            if (has_piece(c)) m_all = fmaxf(m_all, p.slots[(size_t)(bh + c) * AT_SLOT_FLOATS + AT_D * AT_ROWS + row]);
+            if (has_piece(c)) m_all = fmaxf(m_all, p.slots[(size_t)(bh + c) * AT_SLOT_FLOATS + AT_D * AT_LANES + row]);
         float l_all = 0.f, acc[CB_COLS];
 #pragma unroll
         for (int i = 0; i < CB_COLS; ++i) acc[i] = 0.f;
         for (int c = c_first; c <= c_last; ++c) {
             if (!has_piece(c)) continue;
             const float* slot = p.slots + (size_t)(bh + c) * AT_SLOT_FLOATS;
-            const float m = slot[AT_D * AT_ROWS + row];
+            const float m = slot[AT_D * AT_LANES + row];
             if (m == -INFINITY) continue;
             const float wgt = exp2f(m - m_all);
-            l_all = fmaf(slot[AT_D * AT_ROWS + AT_ROWS + row], wgt, l_all);
+            l_all = fmaf(slot[AT_D * AT_LANES + AT_LANES + row], wgt, l_all);
 #pragma unroll
-            for (int i = 0; i < CB_COLS; ++i) acc[i] = fmaf(slot[(size_t)(c0 + i) * AT_ROWS + row], wgt, acc[i]);
+            for (int i = 0; i < CB_COLS; ++i) acc[i] = fmaf(slot[(size_t)(c0 + i) * AT_LANES + row], wgt, acc[i]);
         }
         const float inv = 1.f / l_all;
 #pragma unroll
@@ -761,7 +802,7 @@ __global__ void __launch_bounds__(128) tree_attention_combine_kernel(const AtPar
     // rows x 16 values -> each thread stores 8 consecutive values (16 bytes) of one row
     for (int i = threadIdx.x; i < rows * 2; i += 128) {
         const int r = i >> 1, q8 = (i & 1) * 8;
-        const size_t off = ((size_t)(p.row_off[b] + r) * p.H + h) * AT_D + c0 + q8;
+        const size_t off = ((size_t)(sched.row0[b] + r) * p.H + h) * AT_D + c0 + q8;
         store8_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, &stage[r][q8]);
     }
 }
@@ -781,13 +822,13 @@ EncodeTiledFn at_encode_fn() {
     });
     return fn;
 }
-// bf16 matrix [rows][cols] row-major, boxes of [128 rows][64 cols], 128-byte swizzle, zero fill.
-bool at_make_map(CUtensorMap* map, const void* base_ptr, size_t rows, size_t cols) {
+// bf16 matrix [rows][cols] row-major, boxes of [box_rows][64 cols], 128-byte swizzle, zero fill.
+bool at_make_map(CUtensorMap* map, const void* base_ptr, size_t rows, size_t cols, int box_rows) {
     EncodeTiledFn fn = at_encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {64, 128};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base_ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -796,7 +837,21 @@ bool at_make_map(CUtensorMap* map, const void* base_ptr, size_t rows, size_t col
 
 constexpr int AT_MAX_GRID = 148;
 constexpr int AT_WHOLE_HEAD_TILES = 8;      // up to 1024 keys: heads are handled one by one when B == 1
-constexpr int AT_CLUSTER_MAX_TILES_DEFAULT = 1 << 20;
+
+typedef void (*AtKernel)(CUtensorMap, CUtensorMap, CUtensorMap, AtParams);
+AtKernel at_kernel(bool wide, bool precise) {
+    if (wide) return precise ? tree_attention_tc_kernel<true, true> : tree_attention_tc_kernel<true, false>;
+    return precise ? tree_attention_tc_kernel<false, true> : tree_attention_tc_kernel<false, false>;
+}
+cudaError_t at_set_attributes() {
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] {
+        for (int i = 0; i < 4 && err == cudaSuccess; ++i)
+            err = cudaFuncSetAttribute(at_kernel(i & 1, i >> 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)at_smem(i & 1));
+    });
+    return err;
+}
 
 // How many CTAs may share a head (as one thread-block cluster) when every head is handled on its own: the largest
 // of 4 and 2 for which all H clusters are resident at once, else 1.  Asked of the driver once per head count.
@@ -806,17 +861,17 @@ int at_cluster_size(int H) {
     std::lock_guard<std::mutex> lock(mu);
     if (cached_h == H) return cached_c;
     int pick = 1;
-    if (cudaFuncSetAttribute(tree_attention_tc_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM) == cudaSuccess) {
+    if (at_set_attributes() == cudaSuccess) {
         for (int c = 4; c >= 2 && pick == 1; c /= 2) {
             if (H * c > AT_MAX_GRID) continue;
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(H * c); cfg.blockDim = dim3(at_threads(2)); cfg.dynamicSmemBytes = AT_SMEM;
+            cfg.gridDim = dim3(H * c); cfg.blockDim = dim3(AT_THREADS); cfg.dynamicSmemBytes = at_smem(true);
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr; cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, tree_attention_tc_kernel<2, true>, &cfg) == cudaSuccess && n >= H) pick = c;
+            if (cudaOccupancyMaxActiveClusters(&n, at_kernel(true, true), &cfg) == cudaSuccess && n >= H) pick = c;
         }
     }
     (void)cudaGetLastError();                                // a refused query is not an error of the caller
@@ -824,21 +879,8 @@ int at_cluster_size(int H) {
     return pick;
 }
 
-// Longest prefix (in key tiles) that is still given to clusters.  H clusters of 4 use 4 * H CTAs (128 of the 148 SMs
-// for 32 heads) and need no merge kernel; the contiguous-range shape uses every SM but pays for a second kernel and
-// for the pieces' round trip through memory, which only a long prefix repays.  TRJ_AT_CLUSTER_MAX_TILES overrides
-// the default (a tuning knob, read once).
-int at_cluster_max_tiles() {
-    static const int value = [] {
-        const char* e = getenv("TRJ_AT_CLUSTER_MAX_TILES");
-        const int v = e ? atoi(e) : 0;
-        return v > 0 ? v : AT_CLUSTER_MAX_TILES_DEFAULT;
-    }();
-    return value;
-}
-
 // Launch shape.  The host only knows an upper bound of the key count; CTAs whose range turns out empty do no work.
-struct AtPlan { int grid, cluster; bool merge_kernel; int split; };   // split: threads per query row in the softmax
+struct AtPlan { int grid, cluster; bool merge_kernel; };
 AtPlan at_plan(int32_t B, int32_t H, int32_t max_len) {
     const int tiles_bound = (max_len + AT_KEYS - 1) / AT_KEYS;
     const long long units_bound = (long long)B * H * tiles_bound;
@@ -847,10 +889,10 @@ AtPlan at_plan(int32_t B, int32_t H, int32_t max_len) {
     // Where clusters do not fit, one CTA takes a whole head of up to AT_WHOLE_HEAD_TILES tiles.
     if (B == 1 && H <= AT_MAX_GRID) {
         const int c = tiles_bound >= 2 ? at_cluster_size(H) : 1;
-        if ((c > 1 && tiles_bound <= at_cluster_max_tiles()) || tiles_bound <= AT_WHOLE_HEAD_TILES) return AtPlan{H * c, c, false, 2};
+        if (c > 1 || tiles_bound <= AT_WHOLE_HEAD_TILES) return AtPlan{H * c, c, false};
     }
-    // contiguous ranges + merge kernel; batches of small trees leave row groups empty, so four threads share a row
-    return AtPlan{(int)(units_bound < AT_MAX_GRID ? units_bound : AT_MAX_GRID), 1, true, B > 1 ? 4 : 2};
+    // a batch, or heads too long for one CTA each: all SMs, split as build_range says, and the merge kernel
+    return AtPlan{(int)(units_bound < AT_MAX_GRID ? units_bound : AT_MAX_GRID), 0, true};
 }
 
 }  // namespace
@@ -863,40 +905,32 @@ int timeline_read_attention(int kind, int max_launches, uint64_t* b, uint64_t* e
 int tree_attention_grid(int32_t B, int32_t H, int32_t max_len) { return at_plan(B, H, max_len).grid; }
 
 bool tree_attention_tc_supported(int32_t D, int32_t dtype, int32_t max_rows) {
-    return D == AT_D && dtype == TRJ_BF16 && max_rows <= AT_ROWS && at_encode_fn() != nullptr;
+    return D == AT_D && dtype == TRJ_BF16 && max_rows <= AT_LANES && at_encode_fn() != nullptr;
 }
 
-// Workspace: 256-byte header (status word), then one slot per possible piece: a CTA range can start a
-// new (sequence, head) at most B*H times in total and each of the <= 148 CTAs opens at most one more.
+// Workspace: 256-byte header (status word), then one slot per possible piece: a stream's range can start a
+// new (sequence, head) at most B*H times in total and each of the <= 296 streams opens at most one more.
 size_t tree_attention_tc_workspace(int32_t B, int32_t H) {
-    return 256 + ((size_t)B * H + AT_MAX_GRID) * AT_SLOT_FLOATS * sizeof(float);
+    return 256 + ((size_t)B * H + AT_STREAMS * AT_MAX_GRID) * AT_SLOT_FLOATS * sizeof(float);
 }
 
 cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const void* v_slab, const uint64_t* anc,
                                      int32_t anc_words, const Batch& bt, int32_t H, int32_t Hkv, int32_t max_seq, void* out,
                                      void* out_lo, void* workspace, cudaStream_t st, int* status) {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(tree_attention_tc_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM);
-        if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(tree_attention_tc_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM);
-        if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(tree_attention_tc_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM);
-        if (attr_err == cudaSuccess)
-            attr_err = cudaFuncSetAttribute(tree_attention_tc_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AT_SMEM);
-    });
+    const cudaError_t attr_err = at_set_attributes();
     if (attr_err != cudaSuccess) return attr_err;
+    const bool wide = bt.max_rows > 64;
     CUtensorMap map_q, map_k, map_v;
-    if (!at_make_map(&map_q, q, (size_t)bt.rows_total, (size_t)H * AT_D) ||
-        !at_make_map(&map_k, k_slab, (size_t)(bt.shared_cache ? 1 : bt.B) * Hkv * max_seq, AT_D) ||
-        !at_make_map(&map_v, v_slab, (size_t)(bt.shared_cache ? 1 : bt.B) * Hkv * max_seq, AT_D))
+    if (!at_make_map(&map_q, q, (size_t)bt.rows_total, (size_t)H * AT_D, wide ? 128 : 64) ||
+        !at_make_map(&map_k, k_slab, (size_t)(bt.shared_cache ? 1 : bt.B) * Hkv * max_seq, AT_D, AT_KEYS) ||
+        !at_make_map(&map_v, v_slab, (size_t)(bt.shared_cache ? 1 : bt.B) * Hkv * max_seq, AT_D, AT_KEYS))
         return cudaErrorInvalidValue;
     AtParams p;
     p.seq_len = bt.seq_len; p.row_off = bt.row_off; p.anc = anc; p.anc_words = anc_words;
     p.B = bt.B; p.H = H; p.max_seq = max_seq;
     p.Hkv = Hkv; p.group = H / Hkv;
-    p.early_ok = bt.cached_rows_final;
+    p.in_chain = chain_active();
+    p.early_ok = p.in_chain && bt.cached_rows_final;
     p.shared_cache = bt.shared_cache;
     p.out = (__nv_bfloat16*)out;
     p.out_lo = (__nv_bfloat16*)out_lo;
@@ -906,12 +940,14 @@ cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const vo
     if ((long long)bt.B * H * ((bt.max_len + AT_KEYS - 1) / AT_KEYS) > 0x7fffffffLL) return cudaErrorInvalidValue;   // unit indices are ints
     const AtPlan plan = at_plan(bt.B, H, bt.max_len);
     p.cluster = plan.cluster;
+    p.streams = AT_STREAMS * plan.grid;
+    p.rows_cap = wide ? 128 : 64;
     count_launch();
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.grid); cfg.blockDim = dim3(at_threads(plan.split)); cfg.dynamicSmemBytes = AT_SMEM; cfg.stream = st;
+    cfg.gridDim = dim3(plan.grid); cfg.blockDim = dim3(AT_THREADS); cfg.dynamicSmemBytes = at_smem(wide); cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n_attr = 0;
-    if (chain_active()) {
+    if (pdl_enabled()) {                                     // outside a chain: set up while the previous kernel ends
         attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
         ++n_attr;
@@ -923,20 +959,13 @@ cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const vo
     }
     cfg.attrs = attr; cfg.numAttrs = n_attr;
     // inside a decoder (the caller asks for the result as a bf16 pair) the probabilities are a bf16 pair as well
-    const bool precise = out_lo != nullptr;
-    cudaError_t e;
-    if (plan.split == 4)
-        e = precise ? cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel<4, true>, map_q, map_k, map_v, p)
-                    : cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel<4, false>, map_q, map_k, map_v, p);
-    else
-        e = precise ? cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel<2, true>, map_q, map_k, map_v, p)
-                    : cudaLaunchKernelEx(&cfg, tree_attention_tc_kernel<2, false>, map_q, map_k, map_v, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, at_kernel(wide, out_lo != nullptr), map_q, map_k, map_v, p);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess || !plan.merge_kernel) return e;
     count_launch();
     // The merge kernel's predecessor is always the kernel above, and ahead of its wait it reads only the batch
     // geometry, which was complete before that kernel could start: programmatic launch is safe outside a chain too.
-    e = launch_dependent(pdl_enabled(), tree_attention_combine_kernel, dim3(bt.B * H, AT_D / CB_COLS), dim3(128), 0, st, p, plan.grid);
+    e = launch_dependent(pdl_enabled(), tree_attention_combine_kernel, dim3(bt.B * H, AT_D / CB_COLS), dim3(128), 0, st, p);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -944,7 +973,7 @@ cudaError_t launch_tree_attention(const void* q, const void* k_slab, const void*
                                   int32_t anc_words, const Batch& bt, int32_t H, int32_t Hkv, int32_t D, int32_t max_seq,
                                   int32_t dtype, void* out, void* out_lo, void* workspace, size_t workspace_bytes,
                                   cudaStream_t st, int* status) {
-    if (D == AT_D && dtype == TRJ_BF16 && bt.max_rows <= AT_ROWS) {
+    if (D == AT_D && dtype == TRJ_BF16 && bt.max_rows <= AT_LANES) {
         if (!workspace || ((uintptr_t)workspace % 256) != 0 || workspace_bytes < tree_attention_tc_workspace(bt.B, H) ||
             !tree_attention_tc_supported(D, dtype, bt.max_rows))
             return cudaErrorInvalidValue;
