@@ -52,14 +52,15 @@ class Weights(C.Structure):
 _I32P, _I64P, _U64P = C.POINTER(C.c_int32), C.POINTER(C.c_int64), C.POINTER(C.c_uint64)
 _VP, _I, _SZ = C.c_void_p, C.c_int32, C.c_size_t
 
-# name -> (restype, argtypes); mirrors include/trj.h one to one
+# name -> (restype, argtypes); mirrors include/trj.h one to one.  Host pointers are void pointers here: ctypes passes bytes,
+# ctypes arrays and references as they are, without building a pointer object (1.7 us for a numpy array).
 _SIGNATURES = {
     "trj_last_error": (C.c_char_p, []),
     "trj_version": (C.c_char_p, []),
-    "trj_build_tree": (_I, [_I, _I32P, _I, _I32P, _I, _I, _I, _I, _I32P, _I32P, _I32P, _U64P, _I32P]),
-    "trj_tree_from_parents": (_I, [_I32P, _I, _I, _I32P, _U64P]),
-    "trj_retrieve": (_I, [_I32P, _I, _I, _I, _I64P, _I32P]),
-    "trj_refill_window": (_I, [_I32P, _I32P, _I, _I, _I, _I32P, _I, _I64P, _I32P]),
+    "trj_build_tree": (_I, [_I, _VP, _I, _VP, _I, _I, _I, _I, _VP, _VP, _VP, _VP, _VP]),
+    "trj_tree_from_parents": (_I, [_VP, _I, _I, _VP, _VP]),
+    "trj_retrieve": (_I, [_VP, _I, _I, _I, _VP, _VP]),
+    "trj_refill_window": (_I, [_VP, _VP, _I, _I, _I, _VP, _I, _VP, _VP]),
     "trj_tree_attention_workspace": (_SZ, [_I, _I, _I, _I, _I]),
     "trj_tree_attention": (_I, [_VP, _VP, _VP, _VP, _VP, _VP, _I, _I, _I, _I, _I, _I, _I, _I, _I, _VP, _VP, _SZ, _VP]),
     "trj_tree_attention_gqa": (_I, [_VP, _VP, _VP, _VP, _VP, _VP, _I, _I, _I, _I, _I, _I, _I, _I, _I, _I, _VP, _VP, _SZ, _VP]),
@@ -68,7 +69,7 @@ _SIGNATURES = {
     "trj_topk_accept_workspace": (_SZ, []),
     "trj_topk_accept": (_I, [_VP, _I, _I, _I, _VP, _VP, _VP, _VP, _I, _I, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _SZ, _VP]),
     "trj_node_topk": (_I, [_VP, _I, _I, _VP, _VP]),
-    "trj_refill_tree": (_I, [_I32P, _I32P, _I, _I32P, _I, _I, _I32P, _I, _I64P, _I32P, _I, _I32P]),
+    "trj_refill_tree": (_I, [_VP, _VP, _I, _VP, _I, _I, _VP, _I, _VP, _VP, _I, _VP]),
     "trj_argmax_accept_static": (_I, [_VP, _I, _I, _VP, _VP, _VP, _VP, _I, _I, _VP, _VP, _VP, _VP, _VP, _VP]),
     "trj_compact_rows": (_I, [_VP, _VP, _I, _I, _I, _I, _I, _I, _VP, _VP, _VP, _VP]),
     "trj_workspace_bytes": (_SZ, [C.POINTER(ModelCfg)]),
@@ -83,8 +84,8 @@ _SIGNATURES = {
     "trj_accept": (_I, [_VP, _VP, _VP, _VP, _VP, _I, _I, _VP, _VP, _VP, _VP, _VP]),
     "trj_compact_kv": (_I, [_VP, _VP, _VP, _VP, _I, _VP, _VP, _VP]),
     "trj_prefill": (_I, [_VP, _VP, _VP, _VP, _I, _VP, _I, _VP, _VP]),
-    "trj_step_host": (_I, [_VP, _VP, _VP, _VP, _I, _I, _I32P, _I, _I32P, _I, _I, _I32P, _I32P, _I32P, _I32P,
-                           _I32P, _I32P, _I32P, _VP]),
+    "trj_step_host": (_I, [_VP, _VP, _VP, _VP, _I, _I, _VP, _I, _VP, _I, _I, _VP, _VP, _VP, _VP,
+                           _VP, _VP, _VP, _VP]),
     "trj_draft_tokens": (_I, [_VP, _VP, _VP, _I, _I, _I, _VP, _VP, _VP]),
     "trj_commit_refill": (_I, [_VP, _VP, _VP, _I, _VP, _VP, _VP, _VP, _I, _VP, _I, _VP, _VP, _VP, _VP]),
     "trj_decode_device": (_I, [_VP, _VP, _VP, _VP, _VP, _I, _VP, _I, _VP, _I, _I, _I, _VP, _I, _VP, _VP]),
@@ -218,30 +219,47 @@ def tree_from_parents(parent, anc_words: int = 2) -> Tuple[np.ndarray, np.ndarra
     return depth[:m], anc[:m]
 
 
+def _bytes32(a) -> bytes:
+    return (a if isinstance(a, np.ndarray) and a.dtype == np.int32 else np.asarray(a, np.int32)).tobytes()
+
+
+def _bytes64(a) -> bytes:
+    return (a if isinstance(a, np.ndarray) and a.dtype == np.int64 else np.asarray(a, np.int64)).tobytes()
+
+
+def _out32(n: int):
+    """(ctypes array of n ints for a call to fill, the same memory as a numpy array)."""
+    buf = (C.c_int32 * n)()
+    return buf, np.frombuffer(buf, np.int32)
+
+
 def retrieve(context, n_branches: int, branch_len: int, draws) -> np.ndarray:
     """trj_retrieve: [n_branches, branch_len] retrieved (or noise) tokens."""
-    context = _i32(context)
-    draws = np.ascontiguousarray(draws, dtype=np.int64)
-    out = np.zeros((n_branches, branch_len), np.int32)
-    _check(lib().trj_retrieve(_p32(context), len(context), n_branches, branch_len,
-                              draws.ctypes.data_as(_I64P), _p32(out)))
-    return out
+    context = _bytes32(context)
+    buf, out = _out32(n_branches * branch_len)
+    _check(lib().trj_retrieve(context, len(context) // 4, n_branches, branch_len, _bytes64(draws), buf))
+    return out.reshape(n_branches, branch_len)
 
 
 def refill_window(parent, node_argmax, best: int, width: int, context, draws) -> np.ndarray:
     """trj_refill_window: the next Jacobi window [width]."""
-    parent, node_argmax, context = _i32(parent), _i32(node_argmax), _i32(context)
-    draws = np.ascontiguousarray(draws, dtype=np.int64)
-    out = np.zeros(max(width, 1), np.int32)
-    _check(lib().trj_refill_window(_p32(parent), _p32(node_argmax), len(parent), int(best), width,
-                                   _p32(context), len(context), draws.ctypes.data_as(_I64P), _p32(out)))
+    parent, context = _bytes32(parent), _bytes32(context)
+    buf, out = _out32(max(width, 1))
+    _check(lib().trj_refill_window(parent, _bytes32(node_argmax), len(parent) // 4, int(best), width, context, len(context) // 4,
+                                   _bytes64(draws), buf))
     return out[:width]
 
 
 # ----------------------------------------------------------------------------- device entry points (torch)
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t) -> int:
@@ -262,10 +280,18 @@ def _dev(t, dtype=None, name="tensor"):
     return C.c_void_p(t.data_ptr())
 
 
+def _ptr(t, dtype, name="tensor") -> int:
+    """The address behind a contiguous CUDA tensor of the given type (:func:`_dev` for calls that are made often)."""
+    if getattr(t, "is_cuda", False) and t.dtype is dtype and t.is_contiguous():
+        return t.data_ptr()
+    return _dev(t, dtype, name).value                        # raises, or knows better
+
+
 def _stream(stream=None):
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch()._C                                          # torch.cuda.current_stream() builds a Stream object: 3.2 us
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
 
 
 def _scratch(nbytes: int, device, zero: bool = False):
@@ -286,20 +312,17 @@ def tree_attention(q, k_cache, v_cache, seq_len, row_off, anc, *, max_rows: int,
     torch = _torch()
     rows, n_heads, hd = q.shape
     batch, kv_heads, max_seq, _ = k_cache.shape
+    code = _dtype_code(q)
     if out is None:
         out = torch.empty_like(q)
-    need = tree_attention_workspace(rows, batch, n_heads, hd, max_len)
     if workspace is None:
-        workspace = _scratch(need, q.device)
-    args = (_dev(q, name="q"), _dev(k_cache, q.dtype, "k_cache"), _dev(v_cache, q.dtype, "v_cache"),
-            _dev(seq_len, torch.int32, "seq_len"), _dev(row_off, torch.int32, "row_off"), _dev(anc, torch.int64, "anc"),
-            anc.shape[1], batch, rows, max_rows, n_heads)
-    tail = (hd, max_seq, max_len, _dtype_code(q), _dev(out, q.dtype, "out"), _dev(workspace, torch.uint8, "workspace"),
-            workspace.numel(), _stream(stream))
-    if kv_heads == n_heads:
-        _check(lib().trj_tree_attention(*args, *tail))
-    else:
-        _check(lib().trj_tree_attention_gqa(*args, kv_heads, *tail))
+        workspace = _scratch(tree_attention_workspace(rows, batch, n_heads, hd, max_len), q.device)
+    dt, i32 = q.dtype, torch.int32
+    _check(lib().trj_tree_attention_gqa(
+        _ptr(q, dt, "q"), _ptr(k_cache, dt, "k_cache"), _ptr(v_cache, dt, "v_cache"), _ptr(seq_len, i32, "seq_len"),
+        _ptr(row_off, i32, "row_off"), _ptr(anc, torch.int64, "anc"), anc.shape[1], batch, rows, max_rows, n_heads, kv_heads,
+        hd, max_seq, max_len, code, _ptr(out, dt, "out"), _ptr(workspace, torch.uint8, "workspace"), workspace.numel(),
+        _stream(stream)))
     return out
 
 
@@ -317,16 +340,16 @@ def argmax_accept(logits, tokens, parent, depth, row_off, *, want_margin: bool =
     dev = logits.device
     if workspace is None:
         workspace = _scratch(argmax_accept_workspace(rows, batch), dev, zero=True)
-    i32 = dict(dtype=torch.int32, device=dev)
-    node_argmax = torch.empty(rows, **i32)
+    i32 = torch.int32
+    node_argmax = torch.empty(rows, dtype=i32, device=dev)
     margin = torch.empty(rows, dtype=torch.float32, device=dev) if want_margin else None
-    k_acc, bonus = torch.empty(batch, **i32), torch.empty(batch, **i32)
-    path = torch.empty(batch, PATH_STRIDE, **i32)
+    k_acc, bonus = torch.empty(batch, dtype=i32, device=dev), torch.empty(batch, dtype=i32, device=dev)
+    path = torch.empty(batch, PATH_STRIDE, dtype=i32, device=dev)
     _check(lib().trj_argmax_accept(
-        _dev(logits, name="logits"), _dtype_code(logits), vocab, _dev(tokens, torch.int32, "tokens"),
-        _dev(parent, torch.int32, "parent"), _dev(depth, torch.int32, "depth"), _dev(row_off, torch.int32, "row_off"),
-        batch, rows, _dev(node_argmax), _dev(margin) if want_margin else None, _dev(k_acc), _dev(path), _dev(bonus),
-        _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)))
+        _ptr(logits, logits.dtype, "logits"), _dtype_code(logits), vocab, _ptr(tokens, i32, "tokens"), _ptr(parent, i32, "parent"),
+        _ptr(depth, i32, "depth"), _ptr(row_off, i32, "row_off"), batch, rows, node_argmax.data_ptr(),
+        margin.data_ptr() if want_margin else None, k_acc.data_ptr(), path.data_ptr(), bonus.data_ptr(),
+        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)))
     return {"node_argmax": node_argmax, "margin": margin, "k_acc": k_acc, "path": path, "bonus": bonus}
 
 
@@ -663,30 +686,26 @@ class Model:
 
     def step_host(self, root: int, window, branches, max_len: int, stream=None) -> Dict[str, object]:
         """trj_step_host: one whole decode step from host integers; returns host results."""
-        window = _i32(window).reshape(-1)
-        br = _i32(branches)
-        br = br.reshape(br.shape[0], -1) if br.size else np.zeros((0, 0), np.int32)
-        r, bl = (br.shape[0], br.shape[1]) if br.size else (0, 0)
+        window, br = _bytes32(window), branches if isinstance(branches, np.ndarray) else np.asarray(branches, np.int32)
+        r, bl = (br.shape[0], br.size // br.shape[0]) if br.size else (0, 0)
         hb = self._step_host_buffers()                       # marshalling state that does not change between calls
-        tokens, parent, pred, path = hb["tokens"], hb["parent"], hb["pred"], hb["path"]
         n, k, bonus = hb["n"], hb["k"], hb["bonus"]
-        _check(hb["fn"](self._handle, hb["kc"], hb["vc"], hb["len"], max_len,
-                        int(root), _p32(window), len(window), _p32(br), r, bl, hb["p_tokens"], hb["p_parent"],
-                        hb["r_n"], hb["p_pred"], hb["r_k"], hb["p_path"], hb["r_bonus"], _stream(stream)))
-        m = n.value
-        return {"tokens": tokens[:m].copy(), "parent": parent[:m].copy(), "node_argmax": pred[:m].copy(), "k_acc": k.value,
-                "path": path[:k.value + 1].copy(), "bonus": bonus.value}
+        _check(hb["fn"](self._handle, hb["kc"], hb["vc"], hb["len"], max_len, int(root), window, len(window) // 4, _bytes32(br), r, bl,
+                        hb["c_tokens"], hb["c_parent"], hb["r_n"], hb["c_pred"], hb["r_k"], hb["c_path"], hb["r_bonus"], _stream(stream)))
+        m, acc = n.value, k.value
+        return {"tokens": hb["tokens"][:m].copy(), "parent": hb["parent"][:m].copy(), "node_argmax": hb["pred"][:m].copy(), "k_acc": acc,
+                "path": hb["path"][:acc + 1].copy(), "bonus": bonus.value}
 
     def _step_host_buffers(self):
         hb = getattr(self, "_hb", None)
         if hb is None or hb["ptrs"] != (self.k_cache.data_ptr(), self.v_cache.data_ptr(), self.seq_len.data_ptr()):
-            tokens, parent, pred = (np.zeros(MAX_ROWS, np.int32) for _ in range(3))
-            path = np.zeros(PATH_STRIDE, np.int32)
+            (c_tokens, tokens), (c_parent, parent), (c_pred, pred) = (_out32(MAX_ROWS) for _ in range(3))
+            c_path, path = _out32(PATH_STRIDE)
             n, k, bonus = C.c_int32(0), C.c_int32(0), C.c_int32(0)
             hb = {"ptrs": (self.k_cache.data_ptr(), self.v_cache.data_ptr(), self.seq_len.data_ptr()),
                   "fn": lib().trj_step_host, "kc": _dev(self.k_cache), "vc": _dev(self.v_cache), "len": _dev(self.seq_len),
                   "tokens": tokens, "parent": parent, "pred": pred, "path": path, "n": n, "k": k, "bonus": bonus,
-                  "p_tokens": _p32(tokens), "p_parent": _p32(parent), "p_pred": _p32(pred), "p_path": _p32(path),
+                  "c_tokens": c_tokens, "c_parent": c_parent, "c_pred": c_pred, "c_path": c_path,
                   "r_n": C.byref(n), "r_k": C.byref(k), "r_bonus": C.byref(bonus)}
             self._hb = hb
         return hb
