@@ -58,6 +58,7 @@ struct AtParams {
     __nv_bfloat16* out;          // [rows_total][H][128]
     __nv_bfloat16* out_lo;       // optional: rounding error of `out` as a second bf16 tensor (same shape)
     float* slots;                // partial results, AT_SLOT_FLOATS each
+    int2* owners;                // batches, per (sequence, head): the first and the last stream that worked on it
     int* status;
     float scale_log2;            // log2(e) / sqrt(D)
     int cluster;                 // one sequence: CTAs per thread-block cluster that share one head; 0: a batch
@@ -246,8 +247,10 @@ __device__ __forceinline__ void build_range(Sched& s, const AtParams& p, int cta
             end = begin + s.tiles[b];
         }
     } else {
-        const unsigned U = s.first[p.B], n = p.streams, i = AT_STREAMS * cta + st;
-        if (U < (1u << 22)) {                                // n < 2^9: the products fit 32 bits, whose division is several times cheaper
+        const unsigned U = s.first[p.B], n = min((unsigned)p.streams, U), i = min((unsigned)(AT_STREAMS * cta + st), n);      // every stream below n has a unit
+        if (n == 0 || i == n) {
+            begin = end = (int)U;
+        } else if (U < (1u << 22)) {                                // n < 2^9: the products fit 32 bits, whose division is several times cheaper
             begin = (int)(U * i / n);
             end = (int)(U * (i + 1) / n);
         } else {
@@ -616,6 +619,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_O_FREE + st));
+            if (p.cluster == 0 && stream_thread == 0) {      // for the merge kernel
+                int* const owner = reinterpret_cast<int*>(p.owners + w.bh);
+                if (w.t == 0) owner[0] = AT_STREAMS * (int)blockIdx.x + st;
+                if (w.t + n_tiles == w.tiles) owner[1] = AT_STREAMS * (int)blockIdx.x + st;
+            }
             u += n_tiles;
             ++e;
         }
@@ -749,61 +757,61 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
     TRJ_TL_END(TRJ_TL_ATTENTION);
 }
 
-// Merges the pieces of every (sequence, head) that more than one stream worked on.  One CTA per
-// (sequence, head, 16-wide slice of head_dim), thread = row; pieces are taken in ascending stream order.
-constexpr int CB_COLS = 16;
-__global__ void __launch_bounds__(128) tree_attention_combine_kernel(const AtParams p) {
-    __shared__ Sched sched;
-    __shared__ float stage[AT_LANES][CB_COLS + 1];
-    // the geometry (sequence lengths, row offsets) is not produced by the main kernel: work it out while that
-    // kernel may still be running, and wait for its pieces only afterwards
+// Merges the pieces of every (sequence, head) that more than one stream worked on: one CTA per (sequence, head, 32-wide slice
+// of head_dim), thread = row; pieces are taken in ascending stream order, two at a time so that their loads overlap.  Which
+// streams those are the main kernel has left in p.owners (working the schedule out again in every CTA, with 64-bit
+// divisions, took longer than the merge: a ragged batch of 8 went from 66.5 to 61.7 us, main kernel included).
+constexpr int CB_COLS = 32;
+__global__ void __launch_bounds__(AT_LANES) tree_attention_combine_kernel(const AtParams p) {
+    extern __shared__ float cb_stage[];                      // [row][CB_COLS + 1]
     pdl_launch_dependents();
-    build_batch_sched(sched, p);
-    __syncthreads();
-    if (sched.whole) { pdl_wait(); return; }                 // nothing was split
     const int bh = blockIdx.x, b = bh / p.H, h = bh % p.H, c0 = blockIdx.y * CB_COLS;
-    const long long U = sched.first[p.B];
-    const long long u0 = sched.first[b] + (long long)h * sched.tiles[b], u1 = u0 + sched.tiles[b];
-    if (u0 == u1) { pdl_wait(); return; }                    // a sequence without rows and keys
-    // stream c of the main kernel owns units [U*c/G, U*(c+1)/G): the owner of unit u is the largest c with U*c/G <= u
-    auto owner = [&](long long u) { return (int)(((u + 1) * p.streams + U - 1) / U - 1); };
-    const int c_first = owner(u0), c_last = owner(u1 - 1);
-    const int row = threadIdx.x, rows = sched.rows(b, p.rows_cap);
-    const bool live = row < rows;
-    // a stream in between may own no unit at all (more streams than units): it wrote nothing
-    auto has_piece = [&](int c) {
-        const long long rb = U * c / p.streams, re = U * (c + 1) / p.streams;
-        return (rb > u0 ? rb : u0) < (re < u1 ? re : u1);
-    };
     pdl_wait();
-    if (c_first == c_last) return;                           // written directly by its only stream
-    if (live) {
-        float m_all = -INFINITY;
-        for (int c = c_first; c <= c_last; ++c)
-            if (has_piece(c)) m_all = fmaxf(m_all, p.slots[(size_t)(bh + c) * AT_SLOT_FLOATS + AT_D * AT_LANES + row]);
-        float l_all = 0.f, acc[CB_COLS];
+    const int first_row = p.row_off[b], rows = min(max(p.row_off[b + 1] - first_row, 0), p.rows_cap);
+    const int2 owners = p.owners[bh];
+    if (rows == 0 || owners.x >= owners.y) return;           // written directly by its only stream
+    const int row = threadIdx.x;
+    if (row < rows) {
+        float m_all = -INFINITY, l_all = 0.f, acc[CB_COLS];
 #pragma unroll
         for (int i = 0; i < CB_COLS; ++i) acc[i] = 0.f;
-        for (int c = c_first; c <= c_last; ++c) {
-            if (!has_piece(c)) continue;
-            const float* slot = p.slots + (size_t)(bh + c) * AT_SLOT_FLOATS;
-            const float m = slot[AT_D * AT_LANES + row];
-            if (m == -INFINITY) continue;
-            const float wgt = exp2f(m - m_all);
-            l_all = fmaf(slot[AT_D * AT_LANES + AT_LANES + row], wgt, l_all);
+        for (int c = owners.x; c <= owners.y; c += 2) {
+            float m[2], l[2], o[2][CB_COLS];
 #pragma unroll
-            for (int i = 0; i < CB_COLS; ++i) acc[i] = fmaf(slot[(size_t)(c0 + i) * AT_LANES + row], wgt, acc[i]);
+            for (int j = 0; j < 2; ++j) {
+                if (c + j > owners.y) { m[j] = -INFINITY; continue; }
+                const float* slot = p.slots + (size_t)(bh + c + j) * AT_SLOT_FLOATS;
+                m[j] = slot[AT_D * AT_LANES + row];
+                l[j] = slot[AT_D * AT_LANES + AT_LANES + row];
+#pragma unroll
+                for (int i = 0; i < CB_COLS; ++i) o[j][i] = slot[(size_t)(c0 + i) * AT_LANES + row];
+            }
+            const float m_new = fmaxf(m_all, fmaxf(m[0], m[1]));
+            if (m_new == -INFINITY) continue;                // pieces in which the row sees no key
+            const float keep = exp2f(m_all - m_new);
+            l_all *= keep;
+#pragma unroll
+            for (int i = 0; i < CB_COLS; ++i) acc[i] *= keep;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                if (m[j] == -INFINITY) continue;
+                const float wgt = exp2f(m[j] - m_new);
+                l_all = fmaf(l[j], wgt, l_all);
+#pragma unroll
+                for (int i = 0; i < CB_COLS; ++i) acc[i] = fmaf(o[j][i], wgt, acc[i]);
+            }
+            m_all = m_new;
         }
         const float inv = 1.f / l_all;
 #pragma unroll
-        for (int i = 0; i < CB_COLS; ++i) stage[row][i] = acc[i] * inv;
+        for (int i = 0; i < CB_COLS; ++i) cb_stage[row * (CB_COLS + 1) + i] = acc[i] * inv;
     }
     __syncthreads();
-    // rows x 16 values -> each thread stores 8 consecutive values (16 bytes) of one row
-    for (int i = threadIdx.x; i < rows * 2; i += 128) {
-        const int r = i >> 1, q8 = (i & 1) * 8;
-        const size_t off = ((size_t)(sched.row0[b] + r) * p.H + h) * AT_D + c0 + q8;
-        store8_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, &stage[r][q8]);
+    // each thread stores 8 consecutive values (16 bytes) of one row
+    for (int i = threadIdx.x; i < rows * (CB_COLS / 8); i += blockDim.x) {
+        const int r = i / (CB_COLS / 8), q8 = i % (CB_COLS / 8) * 8;
+        const size_t off = ((size_t)(first_row + r) * p.H + h) * AT_D + c0 + q8;
+        store8_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, cb_stage + r * (CB_COLS + 1) + q8);
     }
 }
 
@@ -908,10 +916,11 @@ bool tree_attention_tc_supported(int32_t D, int32_t dtype, int32_t max_rows) {
     return D == AT_D && dtype == TRJ_BF16 && max_rows <= AT_LANES && at_encode_fn() != nullptr;
 }
 
-// Workspace: 256-byte header (status word), then one slot per possible piece: a stream's range can start a
+// Workspace: 256-byte header (status word), the streams that worked on each (sequence, head), then one slot per possible piece: a stream's range can start a
 // new (sequence, head) at most B*H times in total and each of the <= 296 streams opens at most one more.
+static size_t at_owner_bytes(int32_t B, int32_t H) { return align_up(sizeof(int2) * (size_t)B * H, 256); }
 size_t tree_attention_tc_workspace(int32_t B, int32_t H) {
-    return 256 + ((size_t)B * H + AT_STREAMS * AT_MAX_GRID) * AT_SLOT_FLOATS * sizeof(float);
+    return 256 + at_owner_bytes(B, H) + ((size_t)B * H + AT_STREAMS * AT_MAX_GRID) * AT_SLOT_FLOATS * sizeof(float);
 }
 
 cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const void* v_slab, const uint64_t* anc,
@@ -935,7 +944,8 @@ cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const vo
     p.out = (__nv_bfloat16*)out;
     p.out_lo = (__nv_bfloat16*)out_lo;
     p.status = status ? status : (int*)workspace;
-    p.slots = (float*)((char*)workspace + 256);
+    p.owners = (int2*)((char*)workspace + 256);
+    p.slots = (float*)((char*)workspace + 256 + at_owner_bytes(bt.B, H));
     p.scale_log2 = 1.4426950408889634f / sqrtf((float)AT_D);
     if ((long long)bt.B * H * ((bt.max_len + AT_KEYS - 1) / AT_KEYS) > 0x7fffffffLL) return cudaErrorInvalidValue;   // unit indices are ints
     const AtPlan plan = at_plan(bt.B, H, bt.max_len);
@@ -963,9 +973,9 @@ cudaError_t launch_tree_attention_tc(const void* q, const void* k_slab, const vo
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess || !plan.merge_kernel) return e;
     count_launch();
-    // The merge kernel's predecessor is always the kernel above, and ahead of its wait it reads only the batch
-    // geometry, which was complete before that kernel could start: programmatic launch is safe outside a chain too.
-    e = launch_dependent(pdl_enabled(), tree_attention_combine_kernel, dim3(bt.B * H, AT_D / CB_COLS), dim3(128), 0, st, p);
+    // the merge kernel reads nothing ahead of its wait: programmatic launch is safe outside a chain too
+    e = launch_dependent(pdl_enabled(), tree_attention_combine_kernel, dim3(bt.B * H, AT_D / CB_COLS), dim3(p.rows_cap),
+                         sizeof(float) * p.rows_cap * (CB_COLS + 1), st, p);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -717,15 +717,20 @@ __device__ void accept_sequence(const int32_t* tokens, const int32_t* parent, co
     }
     for (int i = threadIdx.x; i < rows; i += blockDim.x) ok[i] = okb[cur][i];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int best = 0, best_depth = 0;
-        for (int i = 1; i < rows; ++i)
-            if (ok[i] && s_dep[i] > best_depth) { best = i; best_depth = s_dep[i]; }
-        *k_acc = best_depth;
-        *bonus = s_pred[best];
-        int node = best;
-        for (int j = best_depth; j >= 0; --j) { path[j] = node; node = s_par[node]; }
-        s_best = best_depth;
+    if (threadIdx.x < 32) {
+        // the deepest accepted row, the smallest among equals: the largest depth * 128 + (127 - row)
+        unsigned key = TRJ_MAX_ROWS - 1;                     // the root, always accepted
+        for (int i = threadIdx.x; i < rows; i += 32)
+            if (ok[i] && s_dep[i] > 0) key = max(key, (unsigned)s_dep[i] * TRJ_MAX_ROWS + (TRJ_MAX_ROWS - 1 - i));
+        key = __reduce_max_sync(0xffffffffu, key);
+        if (threadIdx.x == 0) {
+            const int best = TRJ_MAX_ROWS - 1 - (int)(key % TRJ_MAX_ROWS), best_depth = (int)(key / TRJ_MAX_ROWS);
+            *k_acc = best_depth;
+            *bonus = s_pred[best];
+            int node = best;
+            for (int j = best_depth; j >= 0; --j) { path[j] = node; node = s_par[node]; }
+            s_best = best_depth;
+        }
     }
     __syncthreads();
     for (int j = s_best + 1 + (int)threadIdx.x; j < TRJ_PATH_STRIDE; j += blockDim.x) path[j] = -1;
@@ -968,15 +973,18 @@ __global__ void __launch_bounds__(TOPK_THREADS) topk_accept_kernel(
 // The arg-max of every verification step (K = 1): one CTA per row, five instructions per element.  A thread scans its
 // elements in ascending id order, so "strictly larger" keeps the smallest id among equals; the runner-up value (for
 // the margin) is max(v2, min(v1, x)).  Threads, then warps, are merged with the full (value, id) order.
-template <typename T>
-__global__ void __launch_bounds__(TOPK_THREADS) argmax_row_accept_kernel(
+// 1024 threads a row up to one row per SM, 512 up to four, else 256: the rows then run in one wave, and what a row waits for
+// (its loads, its reductions, its ticket) is overlapped by the others on its SM.  Rows x 32000 bf16, us per launch with 1024
+// threads and now: 296: 14.4, 9.3; 364: 15.6, 11.9; 700: 27.1, 19.0; 364 x 128256: 31.0, 29.6 (39.6 with 256).
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS) argmax_row_accept_kernel(
         const T* __restrict__ logits, int V, const int32_t* __restrict__ tokens,
         const int32_t* __restrict__ parent, const int32_t* __restrict__ depth,
         const int32_t* __restrict__ row_off, int B, int32_t* node_argmax,
         float* __restrict__ margin, int32_t* __restrict__ k_acc, int32_t* __restrict__ path,
         int32_t* __restrict__ bonus, int do_accept, unsigned int* tickets) {
     pdl_prologue();
-    __shared__ Top red[TOPK_THREADS / 32];
+    __shared__ Top red[THREADS / 32];
     __shared__ int last_flag;
     const int row = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T* lr = logits + (size_t)row * V;
@@ -990,16 +998,16 @@ __global__ void __launch_bounds__(TOPK_THREADS) argmax_row_accept_kernel(
     constexpr int VEC = 16 / (int)sizeof(T);
     if (V % VEC == 0 && ((uintptr_t)logits % 16) == 0) {
         constexpr int BATCH = 4;                             // four 16-byte loads in flight per thread
-        for (int v0 = threadIdx.x * VEC; v0 < V; v0 += BATCH * TOPK_THREADS * VEC) {
+        for (int v0 = threadIdx.x * VEC; v0 < V; v0 += BATCH * THREADS * VEC) {
             uint4 raw[BATCH];
 #pragma unroll
             for (int j = 0; j < BATCH; ++j) {
-                const int v = v0 + j * TOPK_THREADS * VEC;
+                const int v = v0 + j * THREADS * VEC;
                 if (v < V) raw[j] = *reinterpret_cast<const uint4*>(lr + v);
             }
 #pragma unroll
             for (int j = 0; j < BATCH; ++j) {
-                const int v = v0 + j * TOPK_THREADS * VEC;
+                const int v = v0 + j * THREADS * VEC;
                 if (v < V) {
                     const T* e = reinterpret_cast<const T*>(&raw[j]);
 #pragma unroll
@@ -1008,7 +1016,7 @@ __global__ void __launch_bounds__(TOPK_THREADS) argmax_row_accept_kernel(
             }
         }
     } else {
-        for (int v = threadIdx.x; v < V; v += TOPK_THREADS) look(to_f(lr[v]), v);
+        for (int v = threadIdx.x; v < V; v += THREADS) look(to_f(lr[v]), v);
     }
     Top t{v1, i1, v2};
 #pragma unroll
@@ -1016,7 +1024,7 @@ __global__ void __launch_bounds__(TOPK_THREADS) argmax_row_accept_kernel(
     if (lane == 0) red[warp] = t;
     __syncthreads();
     if (warp == 0) {
-        t = red[lane];
+        t = lane < THREADS / 32 ? red[lane] : Top{-INFINITY, 0x7fffffff, -INFINITY};
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t = top_merge(t, top_shfl_xor(t, o));
         if (lane == 0) {
@@ -1335,7 +1343,10 @@ cudaError_t launch_topk_accept(const void* logits, int32_t dtype, int32_t V, int
     cudaError_t launch_err = cudaSuccess;
     unsigned int* tickets = (unsigned int*)ws;
     if (K == 1) {                                            // the step's arg-max: a kernel of its own, five instructions per element
-        DISPATCH_T(dtype, launch_err = launch_chain(argmax_row_accept_kernel<T>, dim3(rows_total), dim3(TOPK_THREADS), 0, st,
+        const int threads = rows_total <= 148 ? 1024 : rows_total <= 4 * 148 ? 512 : 256;
+        DISPATCH_T(dtype, launch_err = launch_chain(threads == 1024 ? argmax_row_accept_kernel<T, 1024>
+                                                    : threads == 512 ? argmax_row_accept_kernel<T, 512> : argmax_row_accept_kernel<T, 256>,
+                                                    dim3(rows_total), dim3(threads), 0, st,
                                                     (const T*)logits, V, tokens, parent, depth, row_off, B, node_argmax,
                                                     margin, k_acc, path, bonus, do_accept ? 1 : 0, tickets));
         if (launch_err == cudaSuccess && topk)

@@ -37,3 +37,24 @@ def test_prompt_cache_rows_and_first_token(trj, dtype, heads, rows):
         assert (np.abs(got - ref) <= tol).all()
     margin = oracle.top2_margin(np.asarray(want)[-1:])[0]
     assert margin < 1e-2 or first == int(oracle.node_argmax(np.asarray(want)[-1:])[0])
+
+
+@pytest.mark.parametrize("rows", [148, 149, 592, 593])
+def test_argmax_of_many_rows(trj, rows):
+    """Either side of the row counts where a row gets fewer threads; ties inside a row, best and runner-up in its last elements."""
+    b, vocab = 8, 1003
+    logits = torch.from_numpy(synth.logits(rows, rows, vocab)).cuda().to(torch.bfloat16)
+    logits[::3, 7] = logits[::3, 900] = 9.0                  # equal maxima: the smaller id
+    logits[1::3, vocab - 1] = 8.0
+    logits[1::3, vocab - 2] = 7.5
+    off = [rows * i // b for i in range(b + 1)]
+    parents = [synth.random_tree(i, off[i + 1] - off[i], 5, 4) for i in range(b)]
+    host = logits.float().cpu().numpy().astype(np.float64)
+    pred = oracle.node_argmax(host)
+    tokens = np.concatenate([synth.planted_tokens(i, p, pred[off[i]:off[i + 1]], vocab) for i, p in enumerate(parents)])
+    got = trj.argmax_accept(logits, i32(tokens), i32(np.concatenate(parents)), i32(np.concatenate([synth.node_depths(p) for p in parents])), i32(off))
+    np.testing.assert_array_equal(got["node_argmax"].cpu().numpy(), pred)
+    np.testing.assert_array_equal(got["margin"].cpu().numpy(), oracle.top2_margin(host).astype(np.float32))
+    for i, p in enumerate(parents):
+        k, path, bonus = oracle.accept_path(tokens[off[i]:off[i + 1]], p, pred[off[i]:off[i + 1]])
+        assert (int(got["k_acc"][i]), got["path"][i, :k + 1].tolist(), int(got["bonus"][i])) == (k, list(path), bonus)
