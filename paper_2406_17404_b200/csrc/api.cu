@@ -394,10 +394,20 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
             char* v_slab = (char*)a.v_cache + ((size_t)l * c.max_batch + a.b0) * seq_stride;
             LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->attn_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
                                                         c.rms_eps, st));
-            LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
-                                          ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
-            LAUNCH(PROF_ROPE, launch_rope_kv_write(pr, ctx->rot, ctx->inv_freq, a.depth, bt, ctx->q, k_slab, v_slab, c.dtype, c.n_heads, Hkv,
-                                                   c.head_dim, c.max_seq, st));
+            // many rows: the projection's epilogue rotates and appends itself
+            if (c.dtype == TRJ_BF16 && c.head_dim == 128 && rotary_table_used(M) && gemm_fuses(M, QKV, d, FusedEpilogue::ROPE)) {
+                FusedEpilogue fe = {};
+                fe.kind = FusedEpilogue::ROPE;
+                fe.q_out = (__nv_bfloat16*)ctx->q; fe.k_slab = (__nv_bfloat16*)k_slab; fe.v_slab = (__nv_bfloat16*)v_slab;
+                fe.H = c.n_heads; fe.Hkv = Hkv; fe.max_seq = c.max_seq; fe.rot = ctx->rot.table; fe.row_at = ctx->rot.row_at;
+                LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
+                                              ctx->gemm_ws_bytes, st, nullptr, nullptr, gemm_status, nullptr, &fe));
+            } else {
+                LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
+                                              ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
+                LAUNCH(PROF_ROPE, launch_rope_kv_write(pr, ctx->rot, ctx->inv_freq, a.depth, bt, ctx->q, k_slab, v_slab, c.dtype, c.n_heads, Hkv,
+                                                       c.head_dim, c.max_seq, st));
+            }
             // inside the decoder the attention result reaches the output projection as a bf16 pair, like every
             // other projection input
             if (!pieces) {
@@ -420,9 +430,17 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
         } else {
             LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->mlp_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
                                                         c.rms_eps, st));
-            LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->w_gate_up[l], ctx->y, M, 2 * c.d_ff, d, c.dtype, ctx->gemm_ws,
-                                          ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
-            LAUNCH(PROF_ELEMENTWISE, launch_swiglu(pr, ctx->act, ctx->act_lo, c.dtype, M, c.d_ff, st));
+            if (c.dtype == TRJ_BF16 && gemm_fuses(M, 2 * c.d_ff, d, FusedEpilogue::SWIGLU)) {      // many rows: SwiGLU in the epilogue
+                FusedEpilogue fe = {};
+                fe.kind = FusedEpilogue::SWIGLU;
+                fe.act = (__nv_bfloat16*)ctx->act; fe.act_lo = (__nv_bfloat16*)ctx->act_lo; fe.f = c.d_ff;
+                LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->w_gate_up[l], ctx->y, M, 2 * c.d_ff, d, c.dtype, ctx->gemm_ws,
+                                              ctx->gemm_ws_bytes, st, nullptr, nullptr, gemm_status, nullptr, &fe));
+            } else {
+                LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->w_gate_up[l], ctx->y, M, 2 * c.d_ff, d, c.dtype, ctx->gemm_ws,
+                                              ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
+                LAUNCH(PROF_ELEMENTWISE, launch_swiglu(pr, ctx->act, ctx->act_lo, c.dtype, M, c.d_ff, st));
+            }
             LAUNCH(PROF_GEMM, launch_gemm(ctx->act, ctx->act_lo, ctx->w_down[l], ctx->y, M, d, c.d_ff, c.dtype, ctx->gemm_ws,
                                           ctx->gemm_ws_bytes, st, out_parts, nullptr, gemm_status));
         }

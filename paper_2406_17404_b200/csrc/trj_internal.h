@@ -124,6 +124,15 @@ inline size_t gemm_top_table_entries(int32_t rows, int32_t N) { return (size_t)r
 // position, [rows][head_dim], and (sequence, cache row) of its K/V.
 struct Rotary { float* table; int2* row_at; };
 bool rotary_table_used(int32_t rows);       // few rows work their rotations out themselves, ahead of their wait
+// What a projection's epilogue does with its finished sums instead of storing them (many rows, bf16, one K range): SwiGLU of a
+// gate/up projection (N = 2 f) into a bf16 pair, or rotary embedding + K/V append of a QKV projection with head_dim 128.
+struct FusedEpilogue {
+    enum Kind { SWIGLU = 1, ROPE = 2 } kind;
+    __nv_bfloat16 *act, *act_lo; int32_t f;                                              // SWIGLU: [rows][f]
+    __nv_bfloat16 *q_out, *k_slab, *v_slab; int32_t H, Hkv, max_seq; const float* rot; const int2* row_at;   // ROPE: as launch_rope_kv_write
+};
+// Whether a projection of this shape with a hi + lo pair of activations is better off with its consumer in the epilogue.
+bool gemm_fuses(int32_t M, int32_t N, int32_t K, FusedEpilogue::Kind kind);
 // h = embedding rows of `tokens`; fills `rot` for the rows of bt (position seq_len[b] + depth[row]).
 cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens, float* h, int32_t d, const double* inv_freq, int32_t D,
                          const int32_t* depth, const Batch& bt, const Rotary& rot, cudaStream_t st);
@@ -143,7 +152,7 @@ size_t gemm_tc_workspace(int32_t M, int32_t N, int32_t K);
 size_t gemm_tc_max_workspace(int32_t max_rows, int32_t N, int32_t K);      // ... of any row count up to max_rows
 cudaError_t launch_gemm_tc(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N, int32_t K,
                            void* workspace, cudaStream_t st, Parts* parts, const WeightPrefetch* ahead = nullptr,
-                           int* status = nullptr, const TopTable* top = nullptr);
+                           int* status = nullptr, const TopTable* top = nullptr, const FusedEpilogue* fused = nullptr);
 // The tcgen05 kernel for every shape it is written for (bf16, K >= 64 and a multiple of 8, N a multiple of 4), the plain
 // kernel for the rest (fp32 models, odd sizes).  A shape of the first kind whose workspace is too small or
 // misaligned is an error (cudaErrorInvalidValue), never a silent detour through the plain kernel.  With `parts`
@@ -153,7 +162,8 @@ cudaError_t launch_gemm_tc(const void* x, const void* x_lo, const void* w, float
 bool gemm_tc_shape(int32_t M, int32_t N, int32_t K, int32_t dtype);
 cudaError_t launch_gemm(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N, int32_t K,
                         int32_t dtype, void* workspace, size_t workspace_bytes, cudaStream_t st, Parts* parts = nullptr,
-                        const WeightPrefetch* ahead = nullptr, int* status = nullptr, const TopTable* top = nullptr);
+                        const WeightPrefetch* ahead = nullptr, int* status = nullptr, const TopTable* top = nullptr,
+                        const FusedEpilogue* fused = nullptr);
 
 // Rotary embedding of q and k at position seq_len[b] + depth[row]; q -> q_out [rows][H][D]; k, v -> cache rows seq_len[b] + local row of the layer slab
 // [B][Hkv][max_seq][D].  The projection result has (H + 2 * Hkv) * D values per row: H query heads, then Hkv key heads, then

@@ -5,7 +5,7 @@ import torch
 
 import oracle
 import synth
-from gpu_util import i32
+from gpu_util import anc_dev, i32
 
 pytestmark = pytest.mark.gpu
 
@@ -58,3 +58,44 @@ def test_argmax_of_many_rows(trj, rows):
     for i, p in enumerate(parents):
         k, path, bonus = oracle.accept_path(tokens[off[i]:off[i + 1]], p, pred[off[i]:off[i + 1]])
         assert (int(got["k_acc"][i]), got["path"][i, :k + 1].tolist(), int(got["bonus"][i])) == (k, list(path), bonus)
+
+
+@pytest.mark.parametrize("rows", [256, 257, 300, 512])
+def test_rotary_and_swiglu_in_the_projections_epilogue(trj, rows):
+    """Either side of one row block of 256: a ragged batch of trees through a decoder whose heads are 128 wide (grouped keys) and
+    whose d_ff ends inside a tile.  K/V rows of every layer (the second layer's rest on the first one's SwiGLU) and logits."""
+    from dataclasses import replace
+    from paper_2406_17404_b200.decode import upload_weights
+    cfg = replace(synth.TINY, dtype="bf16", n_heads=4, n_kv_heads=2, head_dim=128, d_ff=328)
+    layers = [synth.layer_weights(cfg, 4, l) for l in range(cfg.n_layers)]
+    glob = synth.global_weights(cfg, 4)
+    n_seq, prefix = 5, 9
+    model = trj.Model(cfg, *upload_weights(cfg, layers, glob), max_batch=n_seq, max_seq=160, max_rows=128)
+    f64 = lambda d: {k: np.asarray(v, np.float64) for k, v in d.items()}
+    dec = oracle.Decoder(cfg, [f64(l) for l in layers], f64(glob))
+    off = [rows * i // n_seq + (3 if 0 < i < n_seq else 0) for i in range(n_seq + 1)]
+    parents = [synth.random_tree(i, off[i + 1] - off[i], 5, 4) for i in range(n_seq)]
+    tokens = synth.prompt(rows, rows, cfg.vocab)
+    trees = [trj.tree_from_parents(p) for p in parents]
+    words = max(t[1].shape[1] for t in trees)
+    anc = np.concatenate([np.pad(t[1], ((0, 0), (0, words - t[1].shape[1]))) for t in trees])
+    caches = []
+    for b in range(n_seq):
+        prompt = synth.prompt(50 + b, prefix + b, cfg.vocab)
+        model.prefill(i32(prompt), b=b)
+        caches.append(dec.new_cache(160))
+        dec.forward_rows(caches[b], prompt, synth.chain_parents(prefix + b))
+        caches[b].seq_len = prefix + b
+    out = model.verify_step(i32(tokens), i32(np.concatenate(parents)), i32(np.concatenate([t[0] for t in trees])), anc_dev(anc), i32(off),
+                            max_rows=max(np.diff(off)), max_len=prefix + n_seq + max(np.diff(off)), want_logits=True)
+    model.device_status()
+    logits = out["logits"].float().cpu().numpy()
+    for b in range(n_seq):
+        n, m = prefix + b, off[b + 1] - off[b]
+        want = dec.forward_rows(caches[b], tokens[off[b]:off[b + 1]], parents[b])
+        # roundings that fall the other way, as for the prompt above
+        for got, ref in ((model.k_cache, caches[b].k), (model.v_cache, caches[b].v)):
+            got, ref = got[:, b, :, n:n + m].float().cpu().numpy(), np.asarray(ref)[:, :, n:n + m]
+            assert (np.abs(got - ref) <= np.maximum(np.abs(ref), 0.25) * 2.0 ** -7).all()
+            assert float(model.k_cache[:, b, :, n + m:].abs().max()) == 0.0
+        assert np.abs(logits[off[b]:off[b + 1]] - np.asarray(want)).max() <= 2e-2
