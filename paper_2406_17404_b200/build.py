@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -36,6 +37,22 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+CALLS_SRC = os.path.join(HERE, "binding", "calls.cpp")
+CALLS_LIB = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def build_calls(force: bool = False) -> None:
+    """Native callers for the Python binding (host code only).  Without Python's headers the binding stays with ctypes."""
+    header = os.path.join(ROOT, "include", "trj.h")
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")) or not (force or _stale(CALLS_LIB, [CALLS_SRC, header])):
+        return
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", include, "-I", os.path.dirname(header), CALLS_SRC, "-o", CALLS_LIB]
+    r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + r.stdout)
+
+
 def build(verbose: bool = False, force: bool = False, timeline: bool = False, debug: bool = False) -> str:
     """Compile every source under csrc/ and link libtrj.so; returns its path.  ``timeline=True`` builds a second
     library, libtrj_timeline.so, with -DTRJ_TIMELINE (clock stamps in the per-layer kernels; measurement only);
@@ -51,6 +68,7 @@ def build(verbose: bool = False, force: bool = False, timeline: bool = False, de
         finally:
             OBJ, LIB = saved[0], saved[1]
             NVCC_FLAGS[:] = saved[2]
+    build_calls(force)
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(ROOT, "include", "trj.h"))
     if not force and not verbose and not _stale(LIB, [os.path.join(CSRC, s) for s in sources()] + headers):
