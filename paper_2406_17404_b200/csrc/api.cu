@@ -430,7 +430,7 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
         } else {
             LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->mlp_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
                                                         c.rms_eps, st));
-            if (c.dtype == TRJ_BF16 && gemm_fuses(M, 2 * c.d_ff, d, FusedEpilogue::SWIGLU)) {      // many rows: SwiGLU in the epilogue
+            if (c.dtype == TRJ_BF16 && gemm_fuses(M, 2 * c.d_ff, d, FusedEpilogue::SWIGLU)) {      // SwiGLU in the epilogue
                 FusedEpilogue fe = {};
                 fe.kind = FusedEpilogue::SWIGLU;
                 fe.act = (__nv_bfloat16*)ctx->act; fe.act_lo = (__nv_bfloat16*)ctx->act_lo; fe.f = c.d_ff;

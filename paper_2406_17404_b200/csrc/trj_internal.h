@@ -124,8 +124,8 @@ inline size_t gemm_top_table_entries(int32_t rows, int32_t N) { return (size_t)r
 // position, [rows][head_dim], and (sequence, cache row) of its K/V.
 struct Rotary { float* table; int2* row_at; };
 bool rotary_table_used(int32_t rows);       // few rows work their rotations out themselves, ahead of their wait
-// What a projection's epilogue does with its finished sums instead of storing them (many rows, bf16, one K range): SwiGLU of a
-// gate/up projection (N = 2 f) into a bf16 pair, or rotary embedding + K/V append of a QKV projection with head_dim 128.
+// What a projection's epilogue does with its finished sums instead of storing them (bf16, one K range): SwiGLU of a gate/up
+// projection (N = 2 f, f even) into a bf16 pair, or (many rows) rotary embedding + K/V append of a QKV projection with head_dim 128.
 struct FusedEpilogue {
     enum Kind { SWIGLU = 1, ROPE = 2 } kind;
     __nv_bfloat16 *act, *act_lo; int32_t f;                                              // SWIGLU: [rows][f]

@@ -99,3 +99,33 @@ def test_rotary_and_swiglu_in_the_projections_epilogue(trj, rows):
             assert (np.abs(got - ref) <= np.maximum(np.abs(ref), 0.25) * 2.0 ** -7).all()
             assert float(model.k_cache[:, b, :, n + m:].abs().max()) == 0.0
         assert np.abs(logits[off[b]:off[b + 1]] - np.asarray(want)).max() <= 2e-2
+
+
+@pytest.mark.parametrize("rows", [1, 33, 64])
+@pytest.mark.parametrize("d_ff", [9176, 9464, 9472, 9480, 18944, 18952])
+def test_swiglu_of_few_rows_in_the_projections_epilogue(trj, d_ff, rows):
+    """Either side of the range of d_ff whose items fit the grid (31 x 296 < d_ff <= 64 x 296), ragged last items, both
+    ends of the row range: logits of a two-layer decoder."""
+    from dataclasses import replace
+    from paper_2406_17404_b200.decode import upload_weights
+    cfg = replace(synth.TINY, dtype="bf16", n_heads=2, n_kv_heads=2, head_dim=64, d_model=128, d_ff=d_ff)
+    layers = [synth.layer_weights(cfg, 5, l) for l in range(cfg.n_layers)]
+    glob = synth.global_weights(cfg, 5)
+    model = trj.Model(cfg, *upload_weights(cfg, layers, glob), max_batch=1, max_seq=160, max_rows=128)
+    f64 = lambda d: {k: np.asarray(v, np.float64) for k, v in d.items()}
+    dec = oracle.Decoder(cfg, [f64(l) for l in layers], f64(glob))
+    prompt, parent = synth.prompt(7, 9, cfg.vocab), synth.random_tree(rows, rows, min(5, rows - 1), 4) if rows > 1 else np.array([-1], np.int32)
+    tokens = synth.prompt(rows, rows, cfg.vocab)
+    model.prefill(i32(prompt))
+    cache = dec.new_cache(160)
+    dec.forward_rows(cache, prompt, synth.chain_parents(9))
+    cache.seq_len = 9
+    depth, anc = trj.tree_from_parents(parent)
+    out = model.verify_step(i32(tokens), i32(parent), i32(depth), anc_dev(anc), i32([0, rows]), max_rows=rows, max_len=9 + rows, want_logits=True)
+    model.device_status()
+    want = np.asarray(dec.forward_rows(cache, tokens, parent))
+    # the bf16 bound of the model tests: roundings of q and K/V that fall the other way
+    assert np.abs(out["logits"].float().cpu().numpy() - want).max() <= 2e-2
+    got = model.k_cache[:, 0, :, 9:9 + rows].float().cpu().numpy()
+    ref = np.asarray(cache.k)[:, :, 9:9 + rows]
+    assert (np.abs(got - ref) <= np.maximum(np.abs(ref), 0.25) * 2.0 ** -7).all()
