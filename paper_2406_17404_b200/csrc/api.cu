@@ -178,6 +178,7 @@ struct trj_ctx {
     std::vector<const void*> wqkv, wo, w_gate_up, w_down;
     // workspace regions (device)
     float* h; float* y; float* logits;
+    float* h_other; float* y_other; bool small_f32;          // fp32 models: see run_segments
     void* x; void* x_lo; void* q; void* act; void* act_lo;   // *_lo: low halves of split bf16 activations
     double* inv_freq;
     Rotary rot;            // of the rows of the latest forward
@@ -240,6 +241,10 @@ size_t carve(const trj_model_cfg& c, void* ws, trj_ctx* ctx) {
     Carver cv(ws);
     float* h = cv.take<float>((size_t)rows * c.d_model);
     float* y = cv.take<float>((size_t)rows * wide);
+    // fp32 models: second buffers for projections that work out their input themselves, as large as such a product can be
+    const size_t small = c.dtype == TRJ_F32 ? (size_t)SMALL_F32_MAX_TILES * 64 * 64 : 0;
+    float* h_other = cv.take<float>(small);
+    float* y_other = cv.take<float>(small);
     float* logits = cv.take<float>((size_t)step_rows * c.vocab);
     char* x = cv.take<char>((size_t)rows * std::max(c.d_model, HD) * es);
     char* x_lo = cv.take<char>((size_t)rows * std::max(c.d_model, HD) * es);
@@ -272,7 +277,7 @@ size_t carve(const trj_model_cfg& c, void* ws, trj_ctx* ctx) {
     TopEntry* top_table = cv.take<TopEntry>(gemm_top_table_entries(top_rows, c.vocab));
     unsigned int* compact_tickets = cv.take<unsigned int>(TRJ_MAX_BATCH);
     if (ctx) {
-        ctx->h = h; ctx->y = y; ctx->logits = logits; ctx->x = x; ctx->q = q; ctx->act = act;
+        ctx->h = h; ctx->y = y; ctx->h_other = h_other; ctx->y_other = y_other; ctx->logits = logits; ctx->x = x; ctx->q = q; ctx->act = act;
         ctx->x_lo = c.dtype == TRJ_BF16 ? x_lo : nullptr; ctx->act_lo = c.dtype == TRJ_BF16 ? act_lo : nullptr;
         ctx->inv_freq = inv_freq; ctx->rot = Rotary{rot_table, rot_row_at}; ctx->argmax_ws = argmax_ws; ctx->attn_ws = attn_ws; ctx->attn_ws_bytes = attn_bytes;
         ctx->gemm_ws = gemm_ws; ctx->gemm_ws_bytes = gemm_bytes;
@@ -368,10 +373,23 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
     // a quarter); 12-20 MB of the output projection's own weights on top another 0.012 ms, more of them cost again
     constexpr size_t AHEAD_BYTES = (size_t)32 << 20, AHEAD_SELF_BYTES = (size_t)16 << 20;
     const SubChunks* pieces = a.pieces;
+    // Small fp32 models: the projections work out RMSNorm and SwiGLU themselves.  The residual stream then changes between two
+    // buffers, segment by segment, and a projection that reads the latest result of one buffer writes the other one.
+    const bool small = ctx->small_f32 && gemm_small_f32_shape(M, QKV, d) && gemm_small_f32_shape(M, 2 * c.d_ff, d) && gemm_small_f32_shape(M, d, c.d_ff);
+    const auto norm_input = [&](int s, const float* gain, size_t row0) {
+        float* const now = s & 1 ? ctx->h_other : ctx->h;
+        return SmallF32Input{SmallF32Input::NORM, now + row0 * d, pr.ptr ? pr.ptr + row0 * d : nullptr, gain,
+                             s == 2 * c.n_layers ? nullptr : (s & 1 ? ctx->h : ctx->h_other), c.rms_eps};
+    };
     for (int s = s0; s < s1; ++s) {
         const int l = s >> 1;
         Parts* const out_parts = (finish_last && s == s1 - 1) ? nullptr : &pr;
-        if (s == 2 * c.n_layers) {
+        if (s == 2 * c.n_layers && small && gemm_small_f32_shape(a.lm_rows, c.vocab, d)) {
+            ctx->lm_table_rows = 0;
+            if (a.lm_rows > 0)
+                LAUNCH(PROF_GEMM, launch_gemm_small_f32(norm_input(s, ctx->final_norm, a.lm_first), (const float*)ctx->lm_head,
+                                                        pieces ? ctx->logits : ctx->logits + (size_t)a.lm_first * c.vocab, a.lm_rows, c.vocab, d, st));
+        } else if (s == 2 * c.n_layers) {
             LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->final_norm, ctx->x, ctx->x_lo, c.dtype, M, d,
                                                         c.rms_eps, st));
             if (a.lm_rows > 0) {
@@ -392,8 +410,9 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
         } else if ((s & 1) == 0) {
             char* k_slab = (char*)a.k_cache + ((size_t)l * c.max_batch + a.b0) * seq_stride;
             char* v_slab = (char*)a.v_cache + ((size_t)l * c.max_batch + a.b0) * seq_stride;
-            LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->attn_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
-                                                        c.rms_eps, st));
+            if (!small)
+                LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->attn_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
+                                                            c.rms_eps, st));
             // many rows: the projection's epilogue rotates and appends itself
             if (c.dtype == TRJ_BF16 && c.head_dim == 128 && rotary_table_used(M) && gemm_fuses(M, QKV, d, FusedEpilogue::ROPE)) {
                 FusedEpilogue fe = {};
@@ -403,8 +422,13 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
                 LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
                                               ctx->gemm_ws_bytes, st, nullptr, nullptr, gemm_status, nullptr, &fe));
             } else {
-                LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
-                                              ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
+                if (small) {
+                    LAUNCH(PROF_GEMM, launch_gemm_small_f32(norm_input(s, ctx->attn_norm[l], 0), (const float*)ctx->wqkv[l], ctx->y_other, M, QKV, d, st));
+                    pr = Parts{ctx->y_other, 1, 0};
+                } else {
+                    LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wqkv[l], ctx->y, M, QKV, d, c.dtype, ctx->gemm_ws,
+                                                  ctx->gemm_ws_bytes, st, &pr, nullptr, gemm_status));
+                }
                 LAUNCH(PROF_ROPE, launch_rope_kv_write(pr, ctx->rot, ctx->inv_freq, a.depth, bt, ctx->q, k_slab, v_slab, c.dtype, c.n_heads, Hkv,
                                                        c.head_dim, c.max_seq, st));
             }
@@ -427,6 +451,11 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
             const WeightPrefetch ahead{ctx->w_gate_up[l], 2 * c.d_ff, d, AHEAD_BYTES, 2 * std::max(0, ctx->sm_count - attn_grid), AHEAD_SELF_BYTES};
             LAUNCH(PROF_GEMM, launch_gemm(ctx->x, ctx->x_lo, ctx->wo[l], ctx->y, M, d, HD, c.dtype, ctx->gemm_ws,
                                           ctx->gemm_ws_bytes, st, out_parts, &ahead, gemm_status));
+        } else if (small) {
+            LAUNCH(PROF_GEMM, launch_gemm_small_f32(norm_input(s, ctx->mlp_norm[l], 0), (const float*)ctx->w_gate_up[l], ctx->y_other, M, 2 * c.d_ff, d, st));
+            LAUNCH(PROF_GEMM, launch_gemm_small_f32(SmallF32Input{SmallF32Input::SWIGLU, ctx->y_other, nullptr, nullptr, nullptr, 0.f},
+                                                    (const float*)ctx->w_down[l], ctx->y, M, d, c.d_ff, st));
+            if (out_parts) pr = Parts{ctx->y, 1, 0};
         } else {
             LAUNCH(PROF_ELEMENTWISE, launch_add_rmsnorm(ctx->h, pr, ctx->mlp_norm[l], ctx->x, ctx->x_lo, c.dtype, M, d,
                                                         c.rms_eps, st));
@@ -522,6 +551,10 @@ extern "C" trj_status trj_create(const trj_model_cfg* cfg, const trj_weights* w,
         ctx->w_gate_up.push_back(w->w_gate_up[l]); ctx->w_down.push_back(w->w_down[l]);
     }
     carve(*cfg, workspace, ctx);
+    ctx->small_f32 = cfg->dtype == TRJ_F32 && aligned(w->lm_head, 16) && aligned(w->final_norm, 16);
+    for (int l = 0; l < cfg->n_layers; ++l)
+        for (const void* t : {(const void*)w->attn_norm[l], w->wqkv[l], w->wo[l], (const void*)w->mlp_norm[l], w->w_gate_up[l], w->w_down[l]})
+            ctx->small_f32 = ctx->small_f32 && aligned(t, 16);
     ctx->pin_in = ctx->pin_out = nullptr;
     // tables: rotary frequencies and the chain tree used by prefill
     const int half = cfg->head_dim / 2;

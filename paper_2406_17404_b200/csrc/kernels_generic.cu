@@ -327,7 +327,19 @@ constexpr int SF_ROWS = 16, SF_COLS = 8, SF_THREADS = 256, SF_WARPS = SF_THREADS
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
-__global__ void __launch_bounds__(SF_THREADS) gemm_small_f32_kernel(const float* __restrict__ x, const float* __restrict__ w,
+__device__ __forceinline__ float4 silu_mul(const float4& g, const float4& u) {
+    return make_float4(g.x / (1.f + expf(-g.x)) * u.x, g.y / (1.f + expf(-g.y)) * u.y,
+                       g.z / (1.f + expf(-g.z)) * u.z, g.w / (1.f + expf(-g.w)) * u.w);
+}
+// What precedes a projection of the decoder can be its input: every CTA works the few rows out for itself (residual + RMSNorm,
+// or SwiGLU) while they pass into shared memory, which costs less than a kernel of its own in a chain that launches bound:
+// a step of the tiny decoder (2 layers of 256, 11 rows) has 7 of 26 launches less, 93.0 -> 83.1 us.  All loads of a thread come
+// before their first use; row by row and chunk by chunk they made it 102.7 us.  The CTAs of the first columns keep the
+// residual stream, in another buffer, since the rest still read the old one.
+enum { SF_PLAIN = SmallF32Input::PLAIN, SF_NORM = SmallF32Input::NORM, SF_SWIGLU = SmallF32Input::SWIGLU };
+constexpr int SF_MAX_K = 1024;
+template <int IN, int CHUNKS>                // CHUNKS: float4 of a row per lane, K <= 128 CHUNKS
+__global__ void __launch_bounds__(SF_THREADS) gemm_small_f32_kernel(const SmallF32Input in, const float* __restrict__ w,
                                                                     float* __restrict__ y, int M, int N, int K) {
     extern __shared__ __align__(16) float sf_smem[];
     __shared__ float red[SF_WARPS][SF_ROWS * SF_COLS];
@@ -340,9 +352,69 @@ __global__ void __launch_bounds__(SF_THREADS) gemm_small_f32_kernel(const float*
     pdl_launch_dependents();
     for (int c = warp; c < n_cols; c += SF_WARPS)
         for (int i = lane; i < k4; i += 32) cp_async16(ws + c * stride + 4 * i, w + (size_t)(n0 + c) * K + 4 * i);
+    float4 gain[IN == SF_NORM ? CHUNKS : 1];
+    if constexpr (IN == SF_NORM) {
+#pragma unroll
+        for (int t = 0; t < CHUNKS; ++t)
+            if (lane + 32 * t < k4) gain[t] = reinterpret_cast<const float4*>(in.gain)[lane + 32 * t];
+    }
     pdl_wait();
-    for (int r = warp; r < n_rows; r += SF_WARPS)
-        for (int i = lane; i < k4; i += 32) cp_async16(xs + r * stride + 4 * i, x + (size_t)(m0 + r) * K + 4 * i);
+    if constexpr (IN == SF_PLAIN) {
+        for (int r = warp; r < n_rows; r += SF_WARPS)
+            for (int i = lane; i < k4; i += 32) cp_async16(xs + r * stride + 4 * i, in.x + (size_t)(m0 + r) * K + 4 * i);
+    } else {
+        // rows warp and warp + 8, everything of both requested before any of it is used
+        constexpr int ROWS = SF_ROWS / SF_WARPS;
+        const float4* src = reinterpret_cast<const float4*>(in.x) + (size_t)m0 * k4 * (IN == SF_SWIGLU ? 2 : 1);
+        const float4* add = reinterpret_cast<const float4*>(in.add) + (size_t)m0 * k4;
+        float4 v[ROWS][CHUNKS], a[ROWS][CHUNKS];
+#pragma unroll
+        for (int t = 0; t < CHUNKS; ++t) {
+            const int i = lane + 32 * t;
+#pragma unroll
+            for (int e = 0; e < ROWS; ++e) {
+                const int r = warp + SF_WARPS * e;
+                v[e][t] = a[e][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i >= k4 || r >= n_rows) continue;
+                if constexpr (IN == SF_SWIGLU) {
+                    v[e][t] = src[(size_t)r * 2 * k4 + i];
+                    a[e][t] = src[(size_t)r * 2 * k4 + k4 + i];
+                } else {
+                    v[e][t] = src[(size_t)r * k4 + i];
+                    if (in.add) a[e][t] = add[(size_t)r * k4 + i];
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < ROWS; ++e) {
+            const int r = warp + SF_WARPS * e;
+            if (r >= n_rows) break;
+            float inv = 0.f;
+            if constexpr (IN == SF_NORM) {
+                float ss = 0.f;
+#pragma unroll
+                for (int t = 0; t < CHUNKS; ++t) {
+                    float4& h = v[e][t];
+                    h.x += a[e][t].x; h.y += a[e][t].y; h.z += a[e][t].z; h.w += a[e][t].w;
+                    ss += h.x * h.x + h.y * h.y + h.z * h.z + h.w * h.w;
+                }
+                inv = rsqrtf(warp_sum(ss) / (float)K + in.eps);
+            }
+#pragma unroll
+            for (int t = 0; t < CHUNKS; ++t) {
+                const int i = lane + 32 * t;
+                if (i >= k4) break;
+                const float4 h = v[e][t];
+                if constexpr (IN == SF_NORM) {
+                    if (in.h_out && blockIdx.x == 0) reinterpret_cast<float4*>(in.h_out)[(size_t)(m0 + r) * k4 + i] = h;
+                    *reinterpret_cast<float4*>(xs + r * stride + 4 * i) =
+                        make_float4(h.x * inv * gain[t].x, h.y * inv * gain[t].y, h.z * inv * gain[t].z, h.w * inv * gain[t].w);
+                } else {
+                    *reinterpret_cast<float4*>(xs + r * stride + 4 * i) = silu_mul(h, a[e][t]);
+                }
+            }
+        }
+    }
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     // a lane owns rows r, r + 8 and columns c, c + 4; rows and columns past the end read whatever is there and are not stored
@@ -615,10 +687,6 @@ __global__ void swiglu_kernel(const Parts gu, T* __restrict__ act, T* __restrict
 }
 
 // Four columns per thread (f a multiple of 4).
-__device__ __forceinline__ float4 silu_mul(const float4& g, const float4& u) {
-    return make_float4(g.x / (1.f + expf(-g.x)) * u.x, g.y / (1.f + expf(-g.y)) * u.y,
-                       g.z / (1.f + expf(-g.z)) * u.z, g.w / (1.f + expf(-g.w)) * u.w);
-}
 // From split-K pieces.  64 registers, eight CTAs an SM: with 101 the 710 CTAs of a 33-row step take two waves (3.22 against
 // 3.14 ms a step), with 51 or 42 the eight loads of an item no longer fit and go one after the other (3.19, 3.26 ms).
 constexpr int SWIGLU_THREADS = 128, SWIGLU_MAX_CTAS = 2368;
@@ -1222,26 +1290,34 @@ cudaError_t launch_add_rmsnorm(float* h, const Parts& add, const float* gain, vo
 // The small kernel against the tiled one, us per launch at K = 256 by 64 x 64 tiles: 4: 2.1 / 15.6, 22: 6.0 / 18.2, 66: 12.3 /
 // 18.3, 96: 16.6 / 18.3, 132: 21.7 / 18.4 (it reads its operands again for every 16 rows and 8 columns).  K is bounded by the
 // 24 rows of K that a CTA keeps in shared memory.
-constexpr int SMALL_F32_MAX_K = 1024;
-constexpr unsigned SMALL_F32_MAX_TILES = 96;
+bool gemm_small_f32_shape(int32_t M, int32_t N, int32_t K) {
+    return K % 4 == 0 && K <= SF_MAX_K && (int64_t)((N + 63) / 64) * ((M + 63) / 64) <= SMALL_F32_MAX_TILES;
+}
+cudaError_t launch_gemm_small_f32(const SmallF32Input& in, const float* w, float* y, int32_t M, int32_t N, int32_t K, cudaStream_t st) {
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    const auto smem_of = [](int k) { return (size_t)(SF_ROWS + SF_COLS) * (k + 4) * sizeof(float); };
+    std::call_once(once, [&] {
+        for (auto kernel : {gemm_small_f32_kernel<SF_PLAIN, 1>, gemm_small_f32_kernel<SF_NORM, 2>, gemm_small_f32_kernel<SF_NORM, 8>,
+                            gemm_small_f32_kernel<SF_SWIGLU, 8>})
+            if (attr_err == cudaSuccess)
+                attr_err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(SF_MAX_K));
+    });
+    if (attr_err != cudaSuccess) return attr_err;
+    count_launch();
+    auto kernel = in.kind == SmallF32Input::PLAIN ? gemm_small_f32_kernel<SF_PLAIN, 1> : in.kind == SmallF32Input::SWIGLU ? gemm_small_f32_kernel<SF_SWIGLU, 8>
+                  : K <= 256 ? gemm_small_f32_kernel<SF_NORM, 2> : gemm_small_f32_kernel<SF_NORM, 8>;
+    const cudaError_t e = launch_chain(kernel, dim3((N + SF_COLS - 1) / SF_COLS, (M + SF_ROWS - 1) / SF_ROWS), dim3(SF_THREADS), smem_of(K), st, in, w, y, M, N, K);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 cudaError_t launch_gemm_simt(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N,
                              int32_t K, int32_t dtype, cudaStream_t st) {
+    // Few 64 x 64 tiles and a K whose rows fit shared memory: latency is what counts.
+    if (dtype == TRJ_F32 && gemm_small_f32_shape(M, N, K) && ((uintptr_t)x | (uintptr_t)w) % 16 == 0)
+        return launch_gemm_small_f32(SmallF32Input{SmallF32Input::PLAIN, (const float*)x, nullptr, nullptr, nullptr, 0.f}, (const float*)w, y, M, N, K, st);
     count_launch();
     dim3 grid((N + 63) / 64, (M + 63) / 64);
-    // Few 64 x 64 tiles and a K whose rows fit shared memory: latency is what counts.
-    if (dtype == TRJ_F32 && K % 4 == 0 && K <= SMALL_F32_MAX_K && grid.x * grid.y <= SMALL_F32_MAX_TILES &&
-        ((uintptr_t)x | (uintptr_t)w) % 16 == 0) {
-        static std::once_flag once;
-        static cudaError_t attr_err = cudaSuccess;
-        const auto smem_of = [](int k) { return (size_t)(SF_ROWS + SF_COLS) * (k + 4) * sizeof(float); };
-        std::call_once(once, [&] {
-            attr_err = cudaFuncSetAttribute(gemm_small_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(SMALL_F32_MAX_K));
-        });
-        if (attr_err != cudaSuccess) return attr_err;
-        const cudaError_t e = launch_chain(gemm_small_f32_kernel, dim3((N + SF_COLS - 1) / SF_COLS, (M + SF_ROWS - 1) / SF_ROWS), dim3(SF_THREADS),
-                                           smem_of(K), st, (const float*)x, (const float*)w, y, M, N, K);
-        return e != cudaSuccess ? e : cudaGetLastError();
-    }
     DISPATCH_T(dtype, gemm_simt_kernel<T><<<grid, 256, 0, st>>>((const T*)x, (const T*)x_lo, (const T*)w, y, M, N, K));
     return cudaGetLastError();
 }

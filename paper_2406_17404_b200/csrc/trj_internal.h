@@ -141,6 +141,17 @@ cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens
 cudaError_t launch_add_rmsnorm(float* h, const Parts& add, const float* gain, void* x, void* x_lo, int32_t dtype,
                                int32_t rows, int32_t d, float eps, cudaStream_t st);
 // y[M][N] fp32 = (x + x_lo)[M][K] . w[N][K]^T (x_lo may be null), plain shared-memory tiled FMA kernel.
+// fp32 projections of few tiles, and what may precede them in the same launch: x itself; x = rmsnorm(x + add) * gain with the
+// sum left in h_out (another buffer than x; may be null); x = SwiGLU of x as [M][2 K].  16-byte aligned pointers.
+constexpr int SMALL_F32_MAX_TILES = 96;                      // of 64 x 64 outputs
+struct SmallF32Input {
+    enum Kind { PLAIN, NORM, SWIGLU } kind;
+    const float *x, *add, *gain;
+    float* h_out;
+    float eps;
+};
+bool gemm_small_f32_shape(int32_t M, int32_t N, int32_t K);
+cudaError_t launch_gemm_small_f32(const SmallF32Input& in, const float* w, float* y, int32_t M, int32_t N, int32_t K, cudaStream_t st);
 cudaError_t launch_gemm_simt(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N,
                              int32_t K, int32_t dtype, cudaStream_t st);
 // tcgen05 / TMA projection kernel (gemm_sm100.cu): bf16, K >= 64 and a multiple of 8 (rows of 16-byte multiples).  The workspace
