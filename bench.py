@@ -38,10 +38,8 @@ PROMPT = 512
 METRIC = "draft_tokens_verified_per_s"
 UNIT = "tokens/s"
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of ALL 129 projection launches of one step, from an ncu
-# capture of the current projection kernel on a 4-layer model, scaled to 32 layers + the LM head: per layer 443.3 MB
-# (QKV 102.4, output 65.1 incl. 30 MB of gate/up weights that it prefetches and that ncu's serialised timing counts
-# again in the gate/up launch, gate/up 183.2, down 92.6), LM head 263.1 MB.  Set to None whenever that kernel changes.
-GEMM_TRAFFIC_BYTES_PER_STEP = int(32 * 443.3e6 + 263.1e6)
+# capture of the projection kernels.  None whenever they have changed since the last capture, as now: gate/up applies SwiGLU.
+GEMM_TRAFFIC_BYTES_PER_STEP = None
 
 
 def measured_peaks():
@@ -105,12 +103,12 @@ class ClockSampler:
 # --------------------------------------------------------------------------------------- our arm
 def gemm_bytes_per_step(cfg, rows):
     """Algorithmic bytes of all projections of one verification step: every weight once (bf16), the
-    split-bf16 activations in and the fp32 results out."""
+    split-bf16 activations in and the results out (4 bytes each: fp32 sums, or gate/up's split-bf16 SwiGLU)."""
     d, f, hd, v = cfg.d_model, cfg.d_ff, cfg.n_heads * cfg.head_dim, cfg.vocab
-    per_layer = [(3 * hd, d, 2), (d, hd, 2), (2 * f, d, 2), (d, f, 2)]      # (N, K, activation halves)
+    per_layer = [(3 * hd, d, 3 * hd), (d, hd, d), (2 * f, d, f), (d, f, d)]      # (N, K, results per row)
     total = 0
-    for n, k, halves in per_layer:
-        total += cfg.n_layers * (n * k * 2 + rows * k * 2 * halves + rows * n * 4)
+    for n, k, results in per_layer:
+        total += cfg.n_layers * (n * k * 2 + rows * k * 2 * 2 + rows * results * 4)
     total += v * d * 2 + rows * d * 2 * 2 + rows * v * 4
     return total
 
