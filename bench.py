@@ -38,8 +38,10 @@ PROMPT = 512
 METRIC = "draft_tokens_verified_per_s"
 UNIT = "tokens/s"
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of ALL 129 projection launches of one step, from an ncu
-# capture of the projection kernels.  None whenever they have changed since the last capture, as now: gate/up applies SwiGLU.
-GEMM_TRAFFIC_BYTES_PER_STEP = None
+# capture of the current projection kernels on a 4-layer model, scaled to 32 layers + the LM head: per layer 442.0 MB
+# (QKV 102.3, output 66.2 incl. 32 MB of gate/up weights that it prefetches and that ncu's serialised timing counts
+# again in the gate/up launch, gate/up 181.1, down 92.4), LM head 266.0 MB.  Set to None whenever those kernels change.
+GEMM_TRAFFIC_BYTES_PER_STEP = int(32 * 442.0e6 + 266.0e6)
 
 
 def measured_peaks():

@@ -333,7 +333,7 @@ __device__ __forceinline__ float4 silu_mul(const float4& g, const float4& u) {
 }
 // What precedes a projection of the decoder can be its input: every CTA works the few rows out for itself (residual + RMSNorm,
 // or SwiGLU) while they pass into shared memory, which costs less than a kernel of its own in a chain that launches bound:
-// a step of the tiny decoder (2 layers of 256, 11 rows) has 7 of 26 launches less, 93.0 -> 83.1 us.  All loads of a thread come
+// a step of the tiny decoder (2 layers of 256, 11 rows) has 7 of 23 launches less, 93.0 -> 83.1 us.  All loads of a thread come
 // before their first use; row by row and chunk by chunk they made it 102.7 us.  The CTAs of the first columns keep the
 // residual stream, in another buffer, since the rest still read the old one.
 enum { SF_PLAIN = SmallF32Input::PLAIN, SF_NORM = SmallF32Input::NORM, SF_SWIGLU = SmallF32Input::SWIGLU };
@@ -687,8 +687,9 @@ __global__ void swiglu_kernel(const Parts gu, T* __restrict__ act, T* __restrict
 }
 
 // Four columns per thread (f a multiple of 4).
-// From split-K pieces.  64 registers, eight CTAs an SM: with 101 the 710 CTAs of a 33-row step take two waves (3.22 against
-// 3.14 ms a step), with 51 or 42 the eight loads of an item no longer fit and go one after the other (3.19, 3.26 ms).
+// From split-K pieces.  64 registers, eight CTAs an SM: with 101 the 710 CTAs of 33 rows of the 7B shape take two waves (3.22
+// against 3.14 ms a step, measured when that step used this kernel), with 51 or 42 the eight loads of an item no longer fit
+// and go one after the other (3.19, 3.26 ms).
 constexpr int SWIGLU_THREADS = 128, SWIGLU_MAX_CTAS = 2368;
 template <typename T>
 __global__ void __launch_bounds__(SWIGLU_THREADS, 8) swiglu_pieces_kernel(const Parts gu, T* __restrict__ act, T* __restrict__ act_lo, int rows, int f) {
