@@ -25,8 +25,8 @@ def test_small_f32_gemm(trj, m, n, k):
     assert (out[m] == 7.0).all()
 
 
-# K of both norms and of SwiGLU at and past the bound of 1024, one row, a tile of 16 rows and one more, several row tiles, and
-# (128 rows: 2 x 43 tiles of gate/up, 1100 wide: past the bound) the separate kernels
+# K of the norms and of SwiGLU at and past the bound of 1024 (past it: the separate kernels), one row, a tile of 16 rows and
+# one more, several row tiles
 @pytest.mark.parametrize("d_model,d_ff,rows", [(256, 688, 1), (256, 688, 16), (256, 688, 17), (256, 688, 128), (256, 1024, 11),
                                                (256, 1100, 11), (1024, 260, 11), (1032, 260, 11)])
 def test_norm_and_swiglu_inside_the_small_projections(trj, d_model, d_ff, rows):
