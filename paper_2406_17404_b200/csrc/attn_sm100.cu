@@ -27,6 +27,7 @@
 #include "trj_internal.h"
 #include "sm100_common.cuh"
 #include "timeline.cuh"
+#include "piece_range.h"
 
 namespace trj {
 namespace {
@@ -769,7 +770,7 @@ __global__ void __launch_bounds__(AT_LANES) tree_attention_combine_kernel(const 
     pdl_wait();
     const int first_row = p.row_off[b], rows = min(max(p.row_off[b + 1] - first_row, 0), p.rows_cap);
     const int2 owners = p.owners[bh];
-    if (rows == 0 || owners.x >= owners.y) return;           // written directly by its only stream
+    if (rows == 0 || !pieces_to_merge(owners.x, owners.y, p.streams)) return;      // no rows, written directly by its only stream, or no record
     const int row = threadIdx.x;
     if (row < rows) {
         float m_all = -INFINITY, l_all = 0.f, acc[CB_COLS];

@@ -50,3 +50,19 @@ def test_calls_back_to_back_see_each_others_results(trj):
         apart = step(apart)
         torch.cuda.synchronize()
     assert torch.equal(chained, apart)
+
+
+def test_one_workspace_for_batches_of_other_sizes(trj):
+    """The record of who worked on which head, and the pieces, of one batch must not reach the next one: batches of other B and H,
+    split heads in each, through one workspace that starts as garbage."""
+    cases = [AttnCase(trj, 20 + i, h, 128, prefixes, rows, [synth.random_tree(30 + i + j, m, min(6, m - 1), 3) for j, m in enumerate(rows)], "bf16", pad=1)
+             for i, (h, prefixes, rows) in enumerate([(16, [3000, 40, 1], [16, 64, 2]), (4, [900, 1300], [20, 30]), (32, [100, 2500, 7, 600], [33, 9, 70, 12])])]
+    need = max(trj.tree_attention_workspace(sum(c.rows), len(c.rows), c.h, 128, c.max_len) for c in cases)
+    ws = torch.full((need,), 0x7f, dtype=torch.uint8, device="cuda")
+    ws[:256] = 0                                             # the status word
+    apart = [c.run(trj) for c in cases]
+    together = [c.run(trj, workspace=ws) for c in cases + cases]
+    for got, want in zip(together, apart + apart):
+        assert torch.equal(got, want)
+    for c in cases:
+        check_attention(trj, c, heads=[0, c.h - 1])
