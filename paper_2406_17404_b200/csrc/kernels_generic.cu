@@ -1097,7 +1097,7 @@ __global__ void __launch_bounds__(THREADS) argmax_row_accept_kernel(
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t = top_merge(t, top_shfl_xor(t, o));
         if (lane == 0) {
-            node_argmax[row] = t.i1;
+            node_argmax[row] = t.i1 == 0x7fffffff ? 0 : t.i1;      // nothing above -inf: still an id of the vocabulary
             if (margin) margin[row] = t.v1 - t.v2;
             __threadfence();
             const int b = seq_of_row(row_off, B, row);
