@@ -133,7 +133,6 @@ __device__ __forceinline__ void tmem_st16u(uint32_t taddr, const uint32_t* v) {
                    "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
                  : "memory");                                // no wait: pair with tmem_wait_st
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);      // .x (low half) = a
     return *reinterpret_cast<const uint32_t*>(&h);
