@@ -790,7 +790,7 @@ __device__ void accept_sequence(const int32_t* tokens, const int32_t* parent, co
         // the deepest accepted row, the smallest among equals: the largest depth * 128 + (127 - row)
         unsigned key = TRJ_MAX_ROWS - 1;                     // the root, always accepted
         for (int i = threadIdx.x; i < rows; i += 32)
-            if (ok[i] && s_dep[i] > 0) key = max(key, (unsigned)s_dep[i] * TRJ_MAX_ROWS + (TRJ_MAX_ROWS - 1 - i));
+            if (i > 0 && ok[i] && s_dep[i] > 0) key = max(key, (unsigned)s_dep[i] * TRJ_MAX_ROWS + (TRJ_MAX_ROWS - 1 - i));
         key = __reduce_max_sync(0xffffffffu, key);
         if (threadIdx.x == 0) {
             const int best = TRJ_MAX_ROWS - 1 - (int)(key % TRJ_MAX_ROWS), best_depth = (int)(key / TRJ_MAX_ROWS);
