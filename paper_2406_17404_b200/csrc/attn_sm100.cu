@@ -747,6 +747,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
             const size_t off = ((size_t)(sched.row0[0] + row) * p.H + head) * AT_D + (rank * slices + slice) * 32 + 4 * chunk;
             store4_split(p.out + off, p.out_lo ? p.out_lo + off : nullptr, acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
         }
+        __syncwarp();                                        // the loop above ends at different times in a warp's lanes
         if (C > 1) cluster_wait();                           // nobody leaves while its sum may still be copied
         __syncthreads();
     }
