@@ -8,7 +8,7 @@ no fallback: if ``libtrj.so`` is missing or a call fails, an exception is raised
 from __future__ import annotations
 
 import ctypes as C
-import importlib
+import importlib.util
 import os
 from types import SimpleNamespace
 from typing import Dict, List, Optional, Sequence, Tuple
@@ -163,10 +163,8 @@ def lib() -> C.CDLL:
         for name, (res, args) in _SIGNATURES.items():
             fn = getattr(handle, name)
             fn.restype, fn.argtypes = res, args
-        try:
+        if importlib.util.find_spec("._calls", __name__) is not None:        # built: then it has to load
             _calls = importlib.import_module("._calls", __name__)
-        except ImportError:
-            pass
         _lib = handle
     return _lib
 

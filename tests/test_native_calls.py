@@ -1,4 +1,7 @@
 """The native callers of the step's entry points against the same calls through ctypes (host functions, no GPU needed)."""
+import os
+import sysconfig
+
 import numpy as np
 import pytest
 
@@ -6,6 +9,8 @@ import pytest
 @pytest.fixture(params=["native", "ctypes"])
 def binding(request, trj, monkeypatch):
     if request.param == "native":
+        if not os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h")):
+            pytest.skip("no Python headers: the binding stays with ctypes")
         assert trj._calls is not None, "binding/calls.cpp is not built"
     else:
         monkeypatch.setattr(trj, "_calls", None)
@@ -35,3 +40,15 @@ def test_native_arguments_are_checked(trj, binding):
     for bad in [(1.5, 1, 1, 1, None, None), (b"", 1 << 31, 1, 1, None, None), (b"", 1, 1, 1, None, b"written to"), (b"", 1, 1, 1, None)]:
         with pytest.raises((TypeError, OverflowError)):
             call(*bad)
+
+
+def test_a_module_that_is_built_but_does_not_load_is_an_error(trj, monkeypatch):
+    if trj._calls is None:
+        pytest.skip("not built")
+
+    def broken(*_):
+        raise ImportError("undefined symbol")
+    monkeypatch.setattr(trj, "_lib", None)
+    monkeypatch.setattr(trj.importlib, "import_module", broken)
+    with pytest.raises(ImportError, match="undefined symbol"):
+        trj.lib()
