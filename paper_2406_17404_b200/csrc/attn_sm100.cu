@@ -750,6 +750,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
         __syncwarp();                                        // the loop above ends at different times in a warp's lanes
         if (C > 1) cluster_wait();                           // nobody leaves while its sum may still be copied
         __syncthreads();
+        if (abort_flag) {                                    // a wait above gave up: let what its peers were copying here land
+            for (int i = 0; i < 64; ++i) __nanosleep(1000);
+            __syncthreads();
+        }
     }
     if (warp == AT_W_MMA) tmem_dealloc(tmem, 512u);
 #ifdef TRJ_TIMELINE
