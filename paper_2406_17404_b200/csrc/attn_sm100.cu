@@ -183,7 +183,7 @@ struct Sched {
     int row0[TRJ_MAX_BATCH + 1];        // a copy of row_off
     int first[TRJ_MAX_BATCH + 1];       // first unit of each sequence (the launcher checks that the count fits an int)
     int head;                           // one sequence: the head of this CTA's cluster; -1 for a batch
-    int whole;                          // batches: every stream takes at most one (sequence, head), whole
+    int whole;                          // every stream takes at most one (sequence, head), whole: nothing to merge
     int u_begin[AT_STREAMS], u_end[AT_STREAMS];      // this CTA's units
     __device__ int rows(int b, int cap) const { return min(max(row0[b + 1] - row0[b], 0), cap); }
     __device__ void locate(int u, Where& w, int cap) const {
@@ -213,7 +213,10 @@ __device__ __forceinline__ void finish_sched(Sched& s, const AtParams& p) {
         u += s.tiles[b] * p.H;
     }
     s.first[p.B] = u;
-    s.head = -1; s.whole = 0;
+    s.head = -1;
+    // One sequence: only a head of one tile without a cluster is whole; its stream writes the output as in a batch (128 rows without a prefix:
+    // 10.3 -> 8.2 us, the merge of a single piece made the difference).
+    s.whole = p.cluster == 1 && longest <= 1;
     if (p.cluster > 0) return;
     // Whole heads need no merge; equal shares are shorter when a head is much longer than a share.  A merge (pieces to L2 and
     // back in the second kernel) takes about as long as six tiles.
@@ -582,7 +585,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
                 float l_row = 0.f;
 #pragma unroll
                 for (int q = 0; q < PARTS; ++q) l_row += part_sum[st][q][row];       // the same order in every thread
-                if (p.cluster > 0) {
+                if (p.cluster > 0 && !sched.whole) {
                     // a piece of the head: O stays in TMEM until both streams are done (it goes where the ring is)
                     if (live && part == 0) { piece_m[st][row] = m_ref; piece_l[st][row] = l_row; }
                 } else if (w.t == 0 && n_tiles == w.tiles) {
@@ -636,7 +639,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const 
         for (int i = 0; i < 64; ++i) __nanosleep(1000);
         __syncthreads();
     }
-    if (p.cluster > 0) {
+    if (p.cluster > 0 && !sched.whole) {
         // Merge of the head's pieces.  Every CTA of the cluster gets here, with or without pieces, and also after a wait that
         // gave up.  First the CTA adds up its own two pieces; then each CTA gets a quarter (half) of head_dim of every
         // other CTA's sum, by bulk copies into its shared memory, and finishes it.  (Reading all pieces of the

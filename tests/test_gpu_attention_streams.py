@@ -27,7 +27,7 @@ def test_batches(trj, h, hk, prefixes, rows):
     check_attention(trj, case, heads=None if h <= 4 else [0, 1, h // 2, h - 1], seqs=seqs)
 
 
-@pytest.mark.parametrize("s,m", [(0, 1), (127, 1), (128, 64), (63, 65), (900, 64), (900, 65), (2500, 128)])
+@pytest.mark.parametrize("s,m", [(0, 1), (0, 64), (0, 65), (0, 128), (70, 58), (127, 1), (128, 64), (63, 65), (900, 64), (900, 65), (2500, 128)])
 def test_one_sequence(trj, s, m):
     """1 to 21 tiles on the eight streams of a head's cluster; 64 and 65 rows take different kernels."""
     parent = synth.random_tree(s + m, m, min(8, m - 1), 3) if m > 1 else np.array([-1], np.int32)
