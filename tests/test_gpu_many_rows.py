@@ -102,10 +102,10 @@ def test_rotary_and_swiglu_in_the_projections_epilogue(trj, rows):
 
 
 @pytest.mark.parametrize("rows", [1, 33, 64])
-@pytest.mark.parametrize("d_ff", [9176, 9464, 9472, 9480, 18944, 18952])
+@pytest.mark.parametrize("d_ff", [7104, 7112, 9176, 9464, 9472, 9480, 18944, 18952])
 def test_swiglu_of_few_rows_in_the_projections_epilogue(trj, d_ff, rows):
-    """Either side of the range of d_ff whose items fit the grid (31 x 296 < d_ff <= 64 x 296), ragged last items, both
-    ends of the row range: logits of a two-layer decoder."""
+    """Either side of the range of d_ff whose items fit the grid (24 x 296 < d_ff <= 64 x 296: items of 32 to 64 gate rows, in
+    eights; of 32 rows up to 32 x 296), ragged last items, both ends of the row range: logits of a two-layer decoder."""
     from dataclasses import replace
     from paper_2406_17404_b200.decode import upload_weights
     cfg = replace(synth.TINY, dtype="bf16", n_heads=2, n_kv_heads=2, head_dim=64, d_model=128, d_ff=d_ff)
@@ -129,3 +129,25 @@ def test_swiglu_of_few_rows_in_the_projections_epilogue(trj, d_ff, rows):
     got = model.k_cache[:, 0, :, 9:9 + rows].float().cpu().numpy()
     ref = np.asarray(cache.k)[:, :, 9:9 + rows]
     assert (np.abs(got - ref) <= np.maximum(np.abs(ref), 0.25) * 2.0 ** -7).all()
+
+
+@pytest.mark.parametrize("d_ff,rows,fused", [(7104, 1, False), (7112, 1, True), (7112, 40, True), (7112, 41, False), (9472, 40, True), (9472, 41, False),
+                                             (9480, 41, True), (9480, 64, True), (18944, 64, True), (18952, 33, False)])
+def test_which_projections_take_swiglu_into_their_epilogue(trj, d_ff, rows, fused):
+    """By the launches of a step: one less per layer than a decoder whose d_ff is below the range."""
+    from dataclasses import replace
+    from paper_2406_17404_b200.decode import upload_weights
+
+    def launches(f):
+        cfg = replace(synth.TINY, dtype="bf16", n_heads=2, n_kv_heads=2, head_dim=64, d_model=128, d_ff=f)
+        model = trj.Model(cfg, *upload_weights(cfg, [synth.layer_weights(cfg, 5, l) for l in range(cfg.n_layers)], synth.global_weights(cfg, 5)),
+                          max_batch=1, max_seq=160, max_rows=128)
+        parent = synth.chain_parents(rows)
+        depth, anc = trj.tree_from_parents(parent)
+        before = trj.launch_count()
+        model.verify_step(i32(np.arange(rows)), i32(parent), i32(depth), anc_dev(anc), i32([0, rows]), max_rows=rows, max_len=rows)
+        model.device_status()
+        return trj.launch_count() - before, cfg.n_layers
+
+    apart, n_layers = launches(2048)
+    assert launches(d_ff)[0] == apart - (n_layers if fused else 0)
