@@ -370,8 +370,8 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
     const int attn_grid = attn_tc ? tree_attention_grid(bt.B, c.n_heads, bt.max_len) : ctx->sm_count;
     int* const gemm_status = ctx->dev_status, *const attn_status = ctx->dev_status + 1;
     // gate/up + own MB, ms per 33-row step of the 7B shape: none 2.989, 8 + 16 2.962, 16 + 16 2.926, 32 + 16 2.922, 48 + 16 2.957,
-    // 16 + 8 2.940.  The first rows of gate/up over all of K, that is the whole weights of some CTAs: the same bytes as the
-    // first columns of every row, which every CTA would start with, 3.014.
+    // 16 + 8 2.940.  Asked for are the first rows of gate/up over all of K: gate rows only, with SwiGLU in the epilogue half of what
+    // about 100 of its CTAs read.  The same bytes as the first columns of every row, which every CTA would start with: 3.014.
     constexpr size_t AHEAD_BYTES = (size_t)32 << 20, AHEAD_SELF_BYTES = (size_t)16 << 20;
     const SubChunks* pieces = a.pieces;
     // Small fp32 models: the projections work out RMSNorm and SwiGLU themselves.  The residual stream then changes between two

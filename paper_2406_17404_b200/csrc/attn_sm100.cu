@@ -114,15 +114,8 @@ __device__ __forceinline__ void umma8_pv(uint32_t tmem_d, uint32_t tmem_a, uint3
 #undef TRJ_MMA_TS
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
     uint32_t r[32];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    tmem_ld32_nowait(taddr, r);
+    tmem_wait_ld();
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
@@ -269,6 +262,8 @@ __device__ __forceinline__ void build_range(Sched& s, const AtParams& p, int cta
 // number of keys (the output of near-uniform attention is a mean of n values and the rounding errors of its n weights do
 // not average out any faster than it does); inside a deep decoder that error flips the bf16 roundings of the next layers'
 // K/V rows and grows with depth.
+// 640 threads leave 96 registers each.  The kernel of 64-row streams fits; that of 128-row streams (two groups of 32 scores a
+// thread) spills 56 bytes a thread, 68 with PRECISE.
 template <bool WIDE, bool PRECISE>
 __global__ void __launch_bounds__(AT_THREADS, 1) tree_attention_tc_kernel(const __grid_constant__ CUtensorMap map_q,
                                                                           const __grid_constant__ CUtensorMap map_k,

@@ -1043,8 +1043,10 @@ __global__ void __launch_bounds__(TOPK_THREADS) topk_accept_kernel(
 // elements in ascending id order, so "strictly larger" keeps the smallest id among equals; the runner-up value (for
 // the margin) is max(v2, min(v1, x)).  Threads, then warps, are merged with the full (value, id) order.
 // 1024 threads a row up to one row per SM, 512 up to four, else 256: the rows then run in one wave, and what a row waits for
-// (its loads, its reductions, its ticket) is overlapped by the others on its SM.  Rows x 32000 bf16, us per launch with 1024
-// threads and now: 296: 14.4, 9.3; 364: 15.6, 11.9; 700: 27.1, 19.0; 364 x 128256: 31.0, 29.6 (39.6 with 256).
+// (its loads, its reductions, its ticket) is overlapped by the others on its SM.  bf16, us a call with 1024 / 512 / 256 threads: rows x 32000: 64:
+// 7.7 / 7.7 / 8.2, 296: 14.9 / 9.6 / 9.8, 592: 22.6 / 12.8 / 12.8, 700: 24.1 / 14.8 / 15.8, 2000: 70.6 / 33.9 / 31.3; x 128256: 64: 11.3 / 12.1 / 14.4, 296: 23.5 /
+// 18.4 / 19.2, 592: 47.5 / 31.6 / 33.9, 700: 50.3 / 42.4 / 46.9, 1024: 69.4 / 49.1 / 52.6, 2000: 141 / 89 / 88.  fp32 x 128256: 364: 43.6 / 34.2 / 39.3, 593: 69.5 / 58.9 /
+// 52.0, 1500: 154 / 126 / 140.  Where 256 threads are taken 512 are up to 10 % faster for wide vocabularies and 10 - 30 % slower for narrow ones.
 template <typename T, int THREADS>
 __global__ void __launch_bounds__(THREADS) argmax_row_accept_kernel(
         const T* __restrict__ logits, int V, const int32_t* __restrict__ tokens,

@@ -37,8 +37,14 @@ trj_status tree_from_parents_impl(const int32_t* parent, int32_t M, int32_t anc_
 // successor start.  A chain kernel that has started therefore knows that everything enqueued before that
 // embedding is complete, so ahead of its own wait it may read what only earlier work wrote: the batch
 // geometry (seq_len, row_off, depth), weights, and cache rows below seq_len.  Anything written inside the
-// chain is read after the wait.  Outside a chain (the op-level entry points, whose predecessor is
-// unknown) kernels are launched without the attribute, and both instructions do nothing.
+// chain is read after the wait.
+// The op-level entry points have no such fence: their predecessor in the stream is unknown and may have written anything they
+// read, row offsets and lengths included.  Those whose kernels read nothing ahead of their wait are launched programmatically all the same:
+// trj_argmax_accept, trj_topk_accept and trj_compact_rows open a ChainScope for that purpose only, and the tensor-core attention
+// kernel, which is told that it is not in a chain (AtParams::in_chain), sets itself up and waits before its first read.
+// So chain_active() says that the attribute may be set, not that the batch geometry is old: a kernel that reads ahead of its
+// wait must be launched from a forward (forward(), trj_tp_segment) and from nowhere else.  All other op-level kernels are
+// launched without the attribute, and both instructions do nothing.
 bool pdl_enabled();
 void set_pdl(bool on);
 bool chain_active();                      // this thread is inside a ChainScope and PDL is enabled
@@ -140,7 +146,6 @@ cudaError_t launch_embed(const void* embed, int32_t dtype, const int32_t* tokens
 // In bf16 models x is written as a bf16 pair: x (hi) and x_lo (the rounding error of hi); x_lo may be null.
 cudaError_t launch_add_rmsnorm(float* h, const Parts& add, const float* gain, void* x, void* x_lo, int32_t dtype,
                                int32_t rows, int32_t d, float eps, cudaStream_t st);
-// y[M][N] fp32 = (x + x_lo)[M][K] . w[N][K]^T (x_lo may be null), plain shared-memory tiled FMA kernel.
 // fp32 projections of few tiles, and what may precede them in the same launch: x itself; x = rmsnorm(x + add) * gain with the
 // sum left in h_out (another buffer than x; may be null); x = SwiGLU of x as [M][2 K].  16-byte aligned pointers.
 constexpr int SMALL_F32_MAX_TILES = 96;                      // of 64 x 64 outputs
@@ -152,6 +157,7 @@ struct SmallF32Input {
 };
 bool gemm_small_f32_shape(int32_t M, int32_t N, int32_t K);
 cudaError_t launch_gemm_small_f32(const SmallF32Input& in, const float* w, float* y, int32_t M, int32_t N, int32_t K, cudaStream_t st);
+// y[M][N] fp32 = (x + x_lo)[M][K] . w[N][K]^T (x_lo may be null), plain shared-memory tiled FMA kernel; few fp32 tiles as above.
 cudaError_t launch_gemm_simt(const void* x, const void* x_lo, const void* w, float* y, int32_t M, int32_t N,
                              int32_t K, int32_t dtype, cudaStream_t st);
 // tcgen05 / TMA projection kernel (gemm_sm100.cu): bf16, K >= 64 and a multiple of 8 (rows of 16-byte multiples).  The workspace
