@@ -398,7 +398,7 @@ trj_status run_segments(trj_ctx* ctx, const StepArgs& a, int s0, int s1, Parts& 
                 // a verification step keeps every row's logits in place; prefill wants one row and gets it in row 0
                 float* lm_out = pieces ? ctx->logits : ctx->logits + (size_t)a.lm_first * c.vocab;
                 // Eq. 1 needs every row's arg-max, not its logits: when the caller says so and the launch keeps all of
-                // a row's partial sums in one accumulator, the epilogue leaves one candidate per 32 outputs and the
+                // a row's sums in one item, the epilogue leaves one candidate per 32 outputs and the
                 // logits are written only if they are wanted as well
                 const bool table = a.lm_mode != 0 && !pieces && a.lm_first == 0 && a.lm_rows == M && M <= ctx->top_table_rows &&
                                    gemm_top_table_ok(M, c.vocab, d, c.dtype, ctx->x_lo != nullptr);
