@@ -38,10 +38,10 @@ PROMPT = 512
 METRIC = "draft_tokens_verified_per_s"
 UNIT = "tokens/s"
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of ALL 129 projection launches of one step, from an ncu
-# capture of the current projection kernels on a 4-layer model, scaled to 32 layers + the LM head: per layer 442.0 MB
-# (QKV 102.3, output 66.2 incl. 32 MB of gate/up weights that it prefetches and that ncu's serialised timing counts
-# again in the gate/up launch, gate/up 181.1, down 92.4), LM head 266.0 MB.  Set to None whenever those kernels change.
-GEMM_TRAFFIC_BYTES_PER_STEP = int(32 * 442.0e6 + 266.0e6)
+# capture of the current projection kernels on a 4-layer model, scaled to 32 layers + the LM head; None: not captured since those
+# kernels last changed.  The last capture (per layer 442.0 MB, LM head 266.0 MB) was taken before long sums were spread over several
+# accumulators, which adds no loads or stores.
+GEMM_TRAFFIC_BYTES_PER_STEP = None
 
 
 def measured_peaks():
